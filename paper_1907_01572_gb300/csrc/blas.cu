@@ -2,33 +2,51 @@
 // Reductions: every block sums a fixed grid-stride slice, reduces it in a fixed
 // tree order and writes one partial; a single block then sums the partials in
 // index order, so repeated runs give bit-identical results.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <utility>
 
 #include "blas.h"
 
 namespace dg {
 namespace {
 
+// Sum over the block (a power of two of threads, at least 32) in a fixed tree
+// order, returned in every lane of warp 0.  An SM adds two FP64 values per
+// clock, so a warp-wide FP64 addition takes 64 clocks of its quarter of the SM:
+// the tree keeps the additions few, and everything scalar (the sum over blocks,
+// the divisions of the recurrences) is left to one warp.
 __device__ inline double block_sum(double v, double* sh) {
     const int t = threadIdx.x;
     sh[t] = v;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (t < s) sh[t] += sh[t + s];
+    for (int s = blockDim.x / 2; s >= 32; s >>= 1) {
+        if (t < s) sh[t] = v = v + sh[t + s];
         __syncthreads();
     }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+    if (t < 32)
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-__global__ void finalize_kernel(const double* partials, int k, double* out) {
+// Blocks of a reduction over n values: the blocks that hold values, at most
+// kRedBlocks.  (The order of summation is that of kRedBlocks blocks whatever
+// the size -- an absent block's partial sum counts as 0 -- but on the 10^2 to
+// 10^4 values of a coarse level most of those blocks were empty.)
+inline int red_blocks(long long n) {
+    const long long g = (n + kRedThreads - 1) / kRedThreads;
+    return (int)(g < 1 ? 1 : (g > kRedBlocks ? kRedBlocks : g));
+}
+
+__global__ void finalize_kernel(const double* partials, int nb, int k, double* out) {
     __shared__ double sh[kRedThreads];
     for (int j = 0; j < k; ++j) {
         double v = 0.0;
-        for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) v += partials[i * 4 + j];
+        for (int i = threadIdx.x; i < nb; i += blockDim.x) v += partials[i * 4 + j];
         const double s = block_sum(v, sh);
         if (threadIdx.x == 0) out[j] = s;
+        __syncthreads();
     }
 }
 
@@ -47,6 +65,7 @@ __global__ void dots_kernel(DotArgs<T> args, int k, long long n, double* partial
             v += (double)args.a[j][i] * (double)args.b[j][i];
         const double s = block_sum(v, sh);
         if (threadIdx.x == 0) partials[blockIdx.x * 4 + j] = s;
+        __syncthreads();
     }
 }
 
@@ -73,8 +92,8 @@ __global__ void residual_init_kernel(const T* b, const T* y, T* r, T* p, long lo
     if (threadIdx.x == 0) partials[blockIdx.x * 4] = s;
 }
 
-__global__ void sm_init_kernel(SmState* s, const double* rr) {
-    s->rr = rr[0];
+__device__ void sm_init_logic(SmState* s, double rr) {
+    s->rr = rr;
     s->lam = 0.0;
     s->stop = 0;
     s->have_prev = 0;
@@ -83,66 +102,45 @@ __global__ void sm_init_kernel(SmState* s, const double* rr) {
     s->skip = 0;
 }
 
-__device__ void alpha_logic(SmState* s, double v) {
-    s->pAp = v;
-    if (s->stop || !(v > 0.0) || !(s->rr > 0.0) || !isfinite(v)) {
-        s->stop = 1;
-        s->a = 0.0;
-        return;
-    }
-    s->a = s->rr / v;
-}
+// The scalar steps below run on all lanes of one warp: its lanes divide at once
+// what a single thread would divide in turn.
 
-__global__ void sm_alpha_kernel(SmState* s, const double* pAp) {
-    const double v = pAp[0];
-    s->pAp = v;
-    if (s->stop || !(v > 0.0) || !(s->rr > 0.0) || !isfinite(v)) {
-        s->stop = 1;
-        s->a = 0.0;
-        return;
+// alpha = r.r / p.Ap (in every lane); 0 and stop if it is not positive.
+__device__ double alpha_logic(SmState* s, double rr, bool stopped, double pAp, bool& stop) {
+    stop = stopped || !(pAp > 0.0) || !(rr > 0.0) || !isfinite(pAp);
+    const double a = stop ? 0.0 : rr / pAp;
+    if (s != nullptr && (threadIdx.x & 31) == 0) {
+        s->pAp = pAp;
+        s->a = a;
+        if (stop) s->stop = 1;
     }
-    s->a = s->rr / v;
-}
-
-template <typename T>
-__global__ void cg_xr_kernel(const SmState* s, T* x, T* r, const T* p, const T* Ap, long long n, double* partials) {
-    __shared__ double sh[kRedThreads];
-    const bool stop = s->stop != 0;
-    const T a = (T)s->a;
-    double v = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (!stop) {
-            x[i] += a * p[i];
-            const T ri = r[i] - a * Ap[i];
-            r[i] = ri;
-            v += (double)ri * (double)ri;
-        }
-    }
-    const double sum = block_sum(v, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x * 4] = sum;
+    return a;
 }
 
 // Gershgorin bound of row k of the Lanczos tridiagonal built from the CG
 // coefficients (Alg. 5, eq. tridiag): T_kk = 1/a_k + b_{k-1}/a_{k-1},
 // |T_k,k-1| = sqrt(b_{k-1})/a_{k-1}, |T_k,k+1| = sqrt(b_k)/a_k.
-__device__ void beta_logic(SmState* s, double rn) {
-    if (s->stop) return;
-    const double beta = rn / s->rr;
+__device__ void beta_logic(SmState* s, double rn, double beta) {
+    const int lane = threadIdx.x & 31;
+    const double num = lane == 0 ? 1.0 : (lane == 1 ? beta : sqrt(beta));
+    const double q = num / s->a;
+    const double ba = __shfl_sync(0xffffffffu, q, 1), right = __shfl_sync(0xffffffffu, q, 2);
+    if (lane != 0) return;
     s->beta = beta;
     s->rr = rn;
-    double diag = 1.0 / s->a, left = 0.0;
+    double diag = q, left = 0.0;
     if (s->have_prev) {
-        diag += s->b_prev / s->a_prev;
-        left = sqrt(s->b_prev) / s->a_prev;
+        diag += s->diag_prev;
+        left = s->right_prev;
     }
-    const double lk = diag + left + sqrt(beta) / s->a;
+    const double lk = diag + left + right;
     if (isfinite(lk) && lk > s->lam) s->lam = lk;
-    s->a_prev = s->a;
-    s->b_prev = beta;
+    s->diag_prev = ba;
+    s->right_prev = right;
     s->have_prev = 1;
 }
 
-// Last block of a grid: sums partials[i * 4] over the grid's blocks in index order.
+// Sums partials[i * 4] over the grid's blocks; true in warp 0 of the last block to finish.
 __device__ bool last_block_sum(double* partials, unsigned* counter, double* sh, double& total) {
     __shared__ bool last;
     __threadfence();
@@ -154,7 +152,25 @@ __device__ bool last_block_sum(double* partials, unsigned* counter, double* sh, 
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += ((volatile double*)partials)[i * 4];
     total = block_sum(v, sh);
     if (threadIdx.x == 0) *counter = 0u;
-    return true;
+    return threadIdx.x < 32;
+}
+
+// r = p = b - y and the smoother's scalars, in one launch.
+template <typename T>
+__global__ void smooth_init_kernel(SmState* s, const T* b, const T* y, T* r, T* p, long long n, double* partials,
+                                   unsigned* counter) {
+    __shared__ double sh[kRedThreads];
+    double v = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const T ri = b[i] - y[i];
+        r[i] = ri;
+        p[i] = ri;
+        v += (double)ri * (double)ri;
+    }
+    const double t = block_sum(v, sh);
+    if (threadIdx.x == 0) partials[blockIdx.x * 4] = t;
+    double total;
+    if (last_block_sum(partials, counter, sh, total) && threadIdx.x == 0) sm_init_logic(s, total);
 }
 
 template <typename T>
@@ -167,7 +183,8 @@ __global__ void cg_alpha_fused_kernel(SmState* s, const T* p, const T* Ap, long 
     const double b = block_sum(v, sh);
     if (threadIdx.x == 0) partials[blockIdx.x * 4] = b;
     double total;
-    if (last_block_sum(partials, counter, sh, total) && threadIdx.x == 0) alpha_logic(s, total);
+    bool stop;
+    if (last_block_sum(partials, counter, sh, total)) alpha_logic(s, s->rr, s->stop != 0, total, stop);
 }
 
 template <typename T>
@@ -188,25 +205,7 @@ __global__ void cg_update_fused_kernel(SmState* s, T* x, T* r, const T* p, const
     const double b = block_sum(v, sh);
     if (threadIdx.x == 0) partials[blockIdx.x * 4] = b;
     double total;
-    if (last_block_sum(partials, counter, sh, total) && threadIdx.x == 0) beta_logic(s, total);
-}
-
-__global__ void sm_beta_kernel(SmState* s, const double* rr_new) {
-    if (s->stop) return;
-    const double rn = rr_new[0];
-    const double beta = rn / s->rr;
-    s->beta = beta;
-    s->rr = rn;
-    double diag = 1.0 / s->a, left = 0.0;
-    if (s->have_prev) {
-        diag += s->b_prev / s->a_prev;
-        left = sqrt(s->b_prev) / s->a_prev;
-    }
-    const double lk = diag + left + sqrt(beta) / s->a;
-    if (isfinite(lk) && lk > s->lam) s->lam = lk;
-    s->a_prev = s->a;
-    s->b_prev = beta;
-    s->have_prev = 1;
+    if (last_block_sum(partials, counter, sh, total) && !s->stop) beta_logic(s, total, total / s->rr);
 }
 
 template <typename T>
@@ -215,6 +214,121 @@ __global__ void cg_p_kernel(const SmState* s, T* p, const T* r, long long n) {
     const T b = (T)s->beta;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         p[i] = r[i] + b * p[i];
+}
+
+// A whole CG step of the eigenvalue estimate -- alpha, the updates of x and r,
+// beta with the Gershgorin bound, the update of p -- by one thread-block
+// cluster: the vectors' values stay in registers (E per thread) between the
+// phases, and the two dot products are exchanged through distributed shared
+// memory.  Bounded by latency (two cluster barriers, two reductions, the
+// divisions), so it takes the place of three launches where one cluster holds
+// the vectors: a CG step beside its apply took 15.9 us in three launches of
+// kRedBlocks blocks and takes 6.5 us at 1,728 values and 10.8 us at 13,824
+// (15 us in three launches of fewer blocks on 110,592 values).  Past 16,384
+// values a block would sum more than four chunks and the FP64 additions of
+// eight SMs alone would take longer than the launches saved.
+constexpr int kCgCluster = 8, kCgThreads = 2 * kRedThreads, kCgMaxE = 4;
+constexpr int kCgChunks = 2 * kCgCluster * kCgMaxE;   // of kRedThreads values: the blocks of the three-launch form
+
+// Sum of the cluster's values (v[j] the product of value i0 + j step), in the
+// order of the three-launch form, in every lane of warp 0 of every block.
+template <int E>
+__device__ inline double cluster_sum(const double (&v)[E], double (*sh)[kCgThreads], double* part) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x, u = t % kRedThreads, half = t / kRedThreads;
+    double w[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) sh[j][t] = w[j] = v[j];
+    __syncthreads();
+    for (int s = kRedThreads / 2; s >= 32; s >>= 1) {
+        if (u < s)
+#pragma unroll
+            for (int j = 0; j < E; ++j) sh[j][t] = w[j] = w[j] + sh[j][t + s];
+        __syncthreads();
+    }
+    if (u < 32) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            for (int o = 16; o > 0; o >>= 1) w[j] += __shfl_xor_sync(0xffffffffu, w[j], o);
+            if (u < kCgCluster) cl.map_shared_rank(part, u)[2 * kCgCluster * j + 2 * cl.block_rank() + half] = w[j];
+        }
+    }
+    cl.sync();
+    double r = 0.0;
+    if (t < 32) {
+        r = part[t];
+        if (E > 2) r += part[t + 32];
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    }
+    return r;
+}
+
+template <typename T, int E>
+__global__ void __cluster_dims__(kCgCluster, 1, 1) __launch_bounds__(kCgThreads)
+    cg_step_cluster_kernel(SmState* s, T* x, T* r, T* p, const T* Ap, int n) {
+    namespace cg = cooperative_groups;
+    __shared__ double sh[E][kCgThreads], part[2][kCgChunks];
+    __shared__ T coef[2];
+    __shared__ int stop_sh;
+    if (threadIdx.x < 2 * kCgChunks) part[threadIdx.x / kCgChunks][threadIdx.x % kCgChunks] = 0.0;
+    __syncthreads();
+    auto started = cg::this_cluster().barrier_arrive();   // every block runs before its shared memory is written
+    const int i0 = blockIdx.x * kCgThreads + threadIdx.x, step = kCgCluster * kCgThreads;
+    const bool warp0 = threadIdx.x < 32;
+    T pv[E], av[E], rv[E], xv[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const int i = i0 + j * step;
+        const bool in = i < n;
+        pv[j] = in ? p[i] : T(0);
+        av[j] = in ? Ap[i] : T(0);
+        rv[j] = in ? r[i] : T(0);
+        xv[j] = in ? x[i] : T(0);
+    }
+    const double rr = s->rr;
+    const bool stopped = s->stop != 0;
+    double v[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) v[j] = (double)pv[j] * (double)av[j];
+    cg::this_cluster().barrier_wait(std::move(started));
+    const double pAp = cluster_sum<E>(v, sh, part[0]);   // (after its barrier every block has read the scalars)
+    if (warp0) {
+        bool stop;
+        const double a = alpha_logic(blockIdx.x == 0 ? s : nullptr, rr, stopped, pAp, stop);
+        if (threadIdx.x == 0) {
+            coef[0] = (T)a;
+            stop_sh = stop;
+        }
+    }
+    __syncthreads();
+    const bool stop = stop_sh != 0;
+    const T at = coef[0];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        v[j] = 0.0;
+        const int i = i0 + j * step;
+        if (stop || i >= n) continue;
+        rv[j] -= at * av[j];
+        x[i] = xv[j] + at * pv[j];
+        r[i] = rv[j];
+        v[j] = (double)rv[j] * (double)rv[j];
+    }
+    const double rn = cluster_sum<E>(v, sh, part[1]);   // (its barrier also ends every access to remote shared memory)
+    if (stop) return;
+    double beta = 0.0;
+    if (warp0) {
+        beta = rn / rr;
+        if (threadIdx.x == 0) coef[1] = (T)beta;
+    }
+    __syncthreads();
+    const T bt = coef[1];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const int i = i0 + j * step;
+        if (i < n) p[i] = rv[j] + bt * pv[j];
+    }
+    if (warp0 && blockIdx.x == 0) beta_logic(s, rn, beta);
 }
 
 // Chebyshev coefficients of Alg. 4 on [lmax/Lambda, lmax], lmax = scale x lam
@@ -382,8 +496,8 @@ cudaError_t dots(const T* const* a, const T* const* b, int k, long long n, Red r
         args.a[j] = a[j];
         args.b[j] = b[j];
     }
-    dots_kernel<T><<<kRedBlocks, kRedThreads, 0, st>>>(args, k, n, red.partials);
-    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, k, red.out);
+    dots_kernel<T><<<red_blocks(n), kRedThreads, 0, st>>>(args, k, n, red.partials);
+    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, red_blocks(n), k, red.out);
     return cudaGetLastError();
 }
 template cudaError_t dots<double>(const double* const*, const double* const*, int, long long, Red, cudaStream_t);
@@ -417,20 +531,25 @@ cudaError_t cast_f2d(const float* s, double* d, long long n, cudaStream_t st) {
 
 template <typename T>
 cudaError_t residual_init(const T* b, const T* y, T* r, T* p, long long n, Red red, cudaStream_t st) {
-    residual_init_kernel<T><<<kRedBlocks, kRedThreads, 0, st>>>(b, y, r, p, n, red.partials);
-    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, 1, red.out);
+    residual_init_kernel<T><<<red_blocks(n), kRedThreads, 0, st>>>(b, y, r, p, n, red.partials);
+    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, red_blocks(n), 1, red.out);
     return cudaGetLastError();
 }
 template cudaError_t residual_init<double>(const double*, const double*, double*, double*, long long, Red, cudaStream_t);
 template cudaError_t residual_init<float>(const float*, const float*, float*, float*, long long, Red, cudaStream_t);
 
-cudaError_t sm_init(SmState* s, const double* rr, cudaStream_t st) {
-    sm_init_kernel<<<1, 1, 0, st>>>(s, rr);
+template <typename T>
+cudaError_t smooth_init(SmState* s, const T* b, const T* y, T* r, T* p, long long n, Red red, cudaStream_t st) {
+    smooth_init_kernel<T><<<red_blocks(n), kRedThreads, 0, st>>>(s, b, y, r, p, n, red.partials, red.counter);
     return cudaGetLastError();
 }
+template cudaError_t smooth_init<double>(SmState*, const double*, const double*, double*, double*, long long, Red,
+                                         cudaStream_t);
+template cudaError_t smooth_init<float>(SmState*, const float*, const float*, float*, float*, long long, Red,
+                                        cudaStream_t);
 template <typename T>
 cudaError_t cg_alpha_fused(SmState* s, const T* p, const T* Ap, long long n, Red red, cudaStream_t st) {
-    cg_alpha_fused_kernel<T><<<kRedBlocks, kRedThreads, 0, st>>>(s, p, Ap, n, red.partials, red.counter);
+    cg_alpha_fused_kernel<T><<<red_blocks(n), kRedThreads, 0, st>>>(s, p, Ap, n, red.partials, red.counter);
     return cudaGetLastError();
 }
 template cudaError_t cg_alpha_fused<double>(SmState*, const double*, const double*, long long, Red, cudaStream_t);
@@ -438,7 +557,7 @@ template cudaError_t cg_alpha_fused<float>(SmState*, const float*, const float*,
 
 template <typename T>
 cudaError_t cg_update_fused(SmState* s, T* x, T* r, const T* p, const T* Ap, long long n, Red red, cudaStream_t st) {
-    cg_update_fused_kernel<T><<<kRedBlocks, kRedThreads, 0, st>>>(s, x, r, p, Ap, n, red.partials, red.counter);
+    cg_update_fused_kernel<T><<<red_blocks(n), kRedThreads, 0, st>>>(s, x, r, p, Ap, n, red.partials, red.counter);
     return cudaGetLastError();
 }
 template cudaError_t cg_update_fused<double>(SmState*, double*, double*, const double*, const double*, long long, Red,
@@ -446,23 +565,25 @@ template cudaError_t cg_update_fused<double>(SmState*, double*, double*, const d
 template cudaError_t cg_update_fused<float>(SmState*, float*, float*, const float*, const float*, long long, Red,
                                             cudaStream_t);
 
-cudaError_t sm_alpha(SmState* s, const double* pAp, cudaStream_t st) {
-    sm_alpha_kernel<<<1, 1, 0, st>>>(s, pAp);
-    return cudaGetLastError();
-}
 template <typename T>
-cudaError_t cg_xr_update(const SmState* s, T* x, T* r, const T* p, const T* Ap, long long n, Red red, cudaStream_t st) {
-    cg_xr_kernel<T><<<kRedBlocks, kRedThreads, 0, st>>>(s, x, r, p, Ap, n, red.partials);
-    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, 1, red.out);
-    return cudaGetLastError();
+bool cg_step_fits(long long n) {
+    return n <= (long long)kCgCluster * kCgThreads * kCgMaxE;
 }
-template cudaError_t cg_xr_update<double>(const SmState*, double*, double*, const double*, const double*, long long, Red, cudaStream_t);
-template cudaError_t cg_xr_update<float>(const SmState*, float*, float*, const float*, const float*, long long, Red, cudaStream_t);
+template bool cg_step_fits<double>(long long);
+template bool cg_step_fits<float>(long long);
 
-cudaError_t sm_beta(SmState* s, const double* rr_new, cudaStream_t st) {
-    sm_beta_kernel<<<1, 1, 0, st>>>(s, rr_new);
+template <typename T>
+cudaError_t cg_step_cluster(SmState* s, T* x, T* r, T* p, const T* Ap, long long n, cudaStream_t st) {
+    const int m = (int)n, one = kCgCluster * kCgThreads;
+    if (m <= one) cg_step_cluster_kernel<T, 1><<<kCgCluster, kCgThreads, 0, st>>>(s, x, r, p, Ap, m);
+    else if (m <= 2 * one) cg_step_cluster_kernel<T, 2><<<kCgCluster, kCgThreads, 0, st>>>(s, x, r, p, Ap, m);
+    else cg_step_cluster_kernel<T, kCgMaxE><<<kCgCluster, kCgThreads, 0, st>>>(s, x, r, p, Ap, m);
     return cudaGetLastError();
 }
+template cudaError_t cg_step_cluster<double>(SmState*, double*, double*, double*, const double*, long long,
+                                             cudaStream_t);
+template cudaError_t cg_step_cluster<float>(SmState*, float*, float*, float*, const float*, long long, cudaStream_t);
+
 template <typename T>
 cudaError_t cg_p_update(const SmState* s, T* p, const T* r, long long n, cudaStream_t st) {
     cg_p_kernel<T><<<grid_for(n), 256, 0, st>>>(s, p, r, n);
@@ -494,8 +615,8 @@ cudaError_t fcg_dq(const FcgState* f, double* d, double* q, const double* v, con
 }
 cudaError_t fcg_update(const FcgState* f, double* u, double* r, const double* d, const double* q, long long n,
                        Red red, cudaStream_t st) {
-    fcg_update_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(f, u, r, d, q, n, red.partials);
-    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, 1, red.out);
+    fcg_update_kernel<<<red_blocks(n), kRedThreads, 0, st>>>(f, u, r, d, q, n, red.partials);
+    finalize_kernel<<<1, kRedThreads, 0, st>>>(red.partials, red_blocks(n), 1, red.out);
     return cudaGetLastError();
 }
 

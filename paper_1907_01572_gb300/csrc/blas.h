@@ -10,7 +10,7 @@ constexpr int kRedThreads = 256;
 constexpr int kMaxCheb = 64;
 
 struct SmState {        // smoother scalars (device)
-    double rr, rr_new, pAp, a, beta, lam, a_prev, b_prev;
+    double rr, pAp, a, beta, lam, diag_prev, right_prev;   // *_prev: b/a and sqrt(b)/a of the previous step
     int stop, have_prev, skip, pad;
     double ca[kMaxCheb], cb[kMaxCheb];
 };
@@ -41,18 +41,21 @@ template <typename T>
 cudaError_t residual_init(const T* b, const T* y, T* r, T* p, long long n, Red red, cudaStream_t st);
 
 // CGEIGS pieces
-cudaError_t sm_init(SmState* s, const double* rr, cudaStream_t st);
-// Fused CG step, two launches plus the p update: (1) p.Ap and alpha, (2) x, r
+// r = p = b - y; smoother scalars from r.r (one launch)
+template <typename T>
+cudaError_t smooth_init(SmState* s, const T* b, const T* y, T* r, T* p, long long n, Red red, cudaStream_t st);
+// One CG step in one launch, for vectors that one cluster holds (cg_step_fits).
+template <typename T>
+bool cg_step_fits(long long n);
+template <typename T>
+cudaError_t cg_step_cluster(SmState* s, T* x, T* r, T* p, const T* Ap, long long n, cudaStream_t st);
+// Larger vectors: fused CG step, two launches plus the p update: (1) p.Ap and alpha, (2) x, r
 // update with r.r, beta and the Gershgorin bound; the last block to finish
 // sums the per-block partials in index order (same result as dots + finalize).
 template <typename T>
 cudaError_t cg_alpha_fused(SmState* s, const T* p, const T* Ap, long long n, Red red, cudaStream_t st);
 template <typename T>
 cudaError_t cg_update_fused(SmState* s, T* x, T* r, const T* p, const T* Ap, long long n, Red red, cudaStream_t st);
-cudaError_t sm_alpha(SmState* s, const double* pAp, cudaStream_t st);
-template <typename T>
-cudaError_t cg_xr_update(const SmState* s, T* x, T* r, const T* p, const T* Ap, long long n, Red red, cudaStream_t st);
-cudaError_t sm_beta(SmState* s, const double* rr_new, cudaStream_t st);
 template <typename T>
 cudaError_t cg_p_update(const SmState* s, T* p, const T* r, long long n, cudaStream_t st);
 // Chebyshev

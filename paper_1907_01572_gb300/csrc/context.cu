@@ -314,9 +314,14 @@ int smooth_t(dg_ctx* c, int l, const T* b, T* x, const dg_cheb_opts* o) {
     const long long n = c->lv[l].h.n_dofs();
     cudaStream_t st = c->st;
     if ((rc = solver_apply<T>(c, l, x, W.Ap))) return rc;
-    CK(residual_init<T>(b, W.Ap, W.r, W.p, n, c->red, st));
-    CK(sm_init(W.sm, c->red.out, st));
-    c->launches += 3;
+    CK(smooth_init<T>(W.sm, b, W.Ap, W.r, W.p, n, c->red, st));
+    c->launches += 1;
+    const bool one = cg_step_fits<T>(n);
+        if (one) {
+            CK(cg_step_cluster<T>(W.sm, x, W.r, W.p, W.Ap, n, st));
+            c->launches += 1;
+            continue;
+        }
     for (int k = 0; k < ne; ++k) {
         if ((rc = solver_apply<T>(c, l, W.p, W.Ap))) return rc;
         CK(cg_alpha_fused<T>(W.sm, W.p, W.Ap, n, c->red, st));

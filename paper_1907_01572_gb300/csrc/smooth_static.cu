@@ -85,10 +85,14 @@ int smooth_static_t(dg_ctx* c, int l, const T* b, T* x, const dg_cheb_opts* o, u
     const LevelView<T> view = level_view<T>(c, l);
     int launches = 0;
     CKS(launch_apply<T>(view, c->lv[l].buckets, x, Ap, st, &launches));
-    CKS(residual_init<T>(b, Ap, r, p, n, red, st));
-    CKS(sm_init(sm, red.out, st));
+    CKS(smooth_init<T>(sm, b, Ap, r, p, n, red, st));
+    const bool one = cg_step_fits<T>(n);
     for (int k = 0; k < ne; ++k) {
         CKS(launch_apply<T>(view, c->lv[l].buckets, p, Ap, st, &launches));
+        if (one) {
+            CKS(cg_step_cluster<T>(sm, x, r, p, Ap, n, st));
+            continue;
+        }
         CKS(cg_alpha_fused<T>(sm, p, Ap, n, red, st));
         CKS(cg_update_fused<T>(sm, x, r, p, Ap, n, red, st));
         CKS(cg_p_update<T>(sm, p, r, n, st));
@@ -99,7 +103,7 @@ int smooth_static_t(dg_ctx* c, int l, const T* b, T* x, const dg_cheb_opts* o, u
         CKS(launch_apply<T>(view, c->lv[l].buckets, x, Ap, st, &launches));
         CKS(cheb_step<T>(sm, k, b, Ap, p, x, n, st));
     }
-    c->launches += launches + 3 + 3 * ne + 1 + nc;
+    c->launches += launches + 1 + (one ? 1 : 3) * ne + 1 + nc;
     return DG_OK;
 }
 

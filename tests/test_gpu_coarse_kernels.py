@@ -1,0 +1,55 @@
+"""The CG step of the smoother's eigenvalue estimate: one cluster, or three
+launches on longer vectors."""
+import math
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1907_01572_gb300 import dgell, inputs  # noqa: E402
+from tests.gpu_util import single  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _smooth_reference(apply, b, x, ne, nc, Lam=20.0):
+    """Algs. 4-5 in FP64 vector operations around the given operator."""
+    x = x.clone()
+    r = b - apply(x)
+    p, rr, lam, prev = r.clone(), float(r @ r), 0.0, None
+    for _ in range(ne):
+        Ap = apply(p)
+        a = rr / float(p @ Ap)
+        x += a * p
+        r = r - a * Ap
+        new = float(r @ r)
+        beta = new / rr
+        row = 1 / a + math.sqrt(beta) / a + ((prev[1] + math.sqrt(prev[1])) / prev[0] if prev else 0.0)
+        lam, prev, rr = max(lam, row), (a, beta), new
+        p = r + beta * p
+    lo = lam / Lam
+    c, d = 0.5 * (lam - lo), 0.5 * (lam + lo)
+    p, a = torch.zeros_like(x), 0.0
+    for k in range(nc):
+        a = 1 / d if k == 0 else (2 * d / (2 * d * d - c * c) if k == 1 else 1 / (d - a * c * c / 4))
+        p = a * (b - apply(x)) + (a * d - 1) * p
+        x = x + p
+    return x, lam
+
+
+# 8 DOFs; the last vector of one value a thread (4,096) and longer ones up to the cluster's 16,384; beyond it
+@pytest.mark.parametrize("desc", [single(1), single(1, level=3), single(4, level=2), inputs.sweep_mesh(level=2, seed=4, pmax=4),
+                                  single(5, level=2), single(6, level=2)],
+                         ids=["8", "4096", "8000", "hp", "13824", "21952"])
+def test_cg_step_and_estimate(desc):
+    ctx = dgell.Context(desc)
+    n = ctx.level_info()["n_dofs"]
+    g = torch.Generator(device="cuda").manual_seed(n)
+    b = torch.randn(n, dtype=torch.float64, device="cuda", generator=g)
+    x = torch.randn(n, dtype=torch.float64, device="cuda", generator=g)
+    ne = min(6, max(1, n // 4))
+    want, lam = _smooth_reference(lambda v: ctx.apply(v, torch.empty_like(v)), b, x, ne, 5)
+    got_lam = ctx.smooth(b, x, n_eigs=ne, n_cheb=5)
+    # six CG steps amplify the rounding of the dot products (n eps) by at most a few hundred
+    assert abs(got_lam - lam) <= 1e-11 * lam
+    assert float((x - want).norm()) <= 1e-11 * float(want.norm())
