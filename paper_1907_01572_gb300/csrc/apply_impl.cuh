@@ -26,8 +26,8 @@
 // Execution: one warp per element (lanes own pencils / face points, __syncwarp
 // between phases); persistent CTAs stride over the bucket, sized for the most
 // resident warps that shared memory and registers allow; face loops are
-// compiled per mortar size q; FP32 stages every mortar table in shared memory
-// as (Im, Dm) pairs.  Each element of a bucket has a descriptor (offsets and
+// compiled per mortar size q; FP32 stages the mortar tables of sides of the
+// kernel's N in shared memory as (Im, Dm) pairs.  Each element of a bucket has a descriptor (offsets and
 // slot range) and each slot a packed record, so one broadcast load and one
 // load per lane start an element; the next element's descriptor is loaded
 // while the current one runs, and its input and slot records are prefetched
@@ -413,7 +413,7 @@ __device__ __forceinline__ void trace_slot(const LevelView<T>& L, const SlotInfo
             df[k] = acc;
         }
         __syncwarp();
-        const T* M1 = sFT + L.ft.off[N - kMinN][Q - kMinN][s.p0];
+        const T* M1 = sFT + face_tab_off(N, Q, s.p0);
 #pragma unroll
         for (int k0 = 0; k0 < Q * N; k0 += 32) {   // unrolled: a lane's iterations overlap
             const int k = k0 + lane;
@@ -434,7 +434,7 @@ __device__ __forceinline__ void trace_slot(const LevelView<T>& L, const SlotInfo
             N1[k] = sn;
         }
         __syncwarp();
-        const T* M2 = sFT + L.ft.off[N - kMinN][Q - kMinN][s.p1];
+        const T* M2 = sFT + face_tab_off(N, Q, s.p1);
         T* out = mt + 4 * s.goff + 2 * s.side * Q2;
 #pragma unroll
         for (int k0 = 0; k0 < Q2; k0 += 32) {   // unrolled: a lane's iterations overlap
@@ -481,7 +481,7 @@ __device__ __forceinline__ void lift_apply(const LevelView<T>& L, const SlotInfo
         T* X1 = X;
         T* X2 = X1 + Q * N;
         T* X3 = X2 + Q * N;
-        const T* M2 = sFT + L.ft.off[N - kMinN][Q - kMinN][s.p1];
+        const T* M2 = sFT + face_tab_off(N, Q, s.p1);
 #pragma unroll
         for (int k0 = 0; k0 < Q * N; k0 += 32) {   // unrolled: a lane's iterations overlap
             const int k = k0 + lane;
@@ -501,7 +501,7 @@ __device__ __forceinline__ void lift_apply(const LevelView<T>& L, const SlotInfo
             X3[k] = s3v;
         }
         __syncwarp();
-        const T* M1 = sFT + L.ft.off[N - kMinN][Q - kMinN][s.p0];
+        const T* M1 = sFT + face_tab_off(N, Q, s.p0);
 #pragma unroll
         for (int k0 = 0; k0 < N2; k0 += 32) {   // unrolled: a lane's iterations overlap
             const int k = k0 + lane;
@@ -607,11 +607,12 @@ struct Layout {
     static constexpr int EWARP = r4(NR + (3 * NR > EFACE ? 3 * NR : EFACE));
 };
 
-// Values ahead of the per-warp scratch: FP32 mortar tables (staged) and the
-// element's 1-D volume tables.
-template <int N>
-__host__ __device__ constexpr int table_vals(int ftot) {
-    return r4(ftot) + vol_vals(N);
+// Values ahead of the per-warp scratch: the mortar tables of sides of this N
+// (FP32 only: at most 1,080 values of the 6,660 of all N; FP64 reads them
+// through L1, measured 1-2 % faster) and the element's 1-D volume tables.
+template <typename T>
+__host__ __device__ constexpr int table_vals(int n) {
+    return (sizeof(T) == 4 ? r4(face_seg_vals(n)) : 0) + vol_vals(n);
 }
 
 // One mortar slot of an element, packed so that a warp can hold the records of
@@ -704,19 +705,20 @@ struct WarpSlots {
     }
 };
 
-// Shared-memory preamble common to both kernels: mortar tables (FP32) and the
-// element's 1-D volume tables; returns the first per-warp scratch value.
+// Shared-memory preamble common to both kernels: the mortar tables of sides of
+// this N and the element's 1-D volume tables; returns the first per-warp
+// scratch value.
 template <int N, typename T>
 __device__ __forceinline__ T* load_tables(const LevelView<T>& L, const T*& sFT, const T*& sI, const T*& sDg,
                                           const T*& sDL) {
-    constexpr bool STAGE = sizeof(T) == 4;
+    constexpr int FTOT = sizeof(T) == 4 ? face_seg_vals(N) : 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
-    const int ftot = STAGE ? L.ft.total : 0;
     T* sFTs = sm;
-    sFT = STAGE ? sFTs : L.ftab;
-    T* sV = sFTs + r4(ftot);
-    for (int k = threadIdx.x; k < ftot; k += blockDim.x) sFTs[k] = L.ftab[k];
+    const T* ftab = L.ftab + face_seg_off(N);
+    sFT = FTOT > 0 ? sFTs : ftab;
+    T* sV = sFTs + r4(FTOT);
+    for (int k = threadIdx.x; k < FTOT; k += blockDim.x) sFTs[k] = ftab[k];
     constexpr int NP = r4(N);
     const T* tI = L.tab + tab_n(TabIndex::I, N);
     const T* tD = L.tab + tab_n(TabIndex::Dg, N);
@@ -1148,9 +1150,9 @@ inline int grid_cap() {
 template <int N, typename T, typename TX, bool OR>
 cudaError_t launch_trace(const LevelView<T>& L, const BucketInfo& b, const TX* x, cudaStream_t st) {
     using Ly = Layout<N>;
-    static const LaunchShape shp = [&] {   // the mortar tables have the same size in every context
+    static const LaunchShape shp = [] {
         LaunchShape r{};
-        const size_t table_bytes = table_vals<N>(sizeof(T) == 4 ? L.ft.total : 0) * sizeof(T);
+        const size_t table_bytes = table_vals<T>(N) * sizeof(T);
         r.err = pick_warps(trace_kernel<N, T, TX, OR>, table_bytes, Ly::TWARP * sizeof(T), r.W, r.smem, r.per_sm);
         return r;
     }();
@@ -1166,9 +1168,9 @@ cudaError_t launch_trace(const LevelView<T>& L, const BucketInfo& b, const TX* x
 template <int N, typename T, typename TX, bool OR, bool BD = false>
 cudaError_t launch_element(const LevelView<T>& L, const BucketInfo& b, const TX* x, T* y, cudaStream_t st) {
     using Ly = Layout<N>;
-    static const LaunchShape shp = [&] {   // the mortar tables have the same size in every context
+    static const LaunchShape shp = [] {
         LaunchShape r{};
-        const size_t table_bytes = table_vals<N>(sizeof(T) == 4 ? L.ft.total : 0) * sizeof(T);
+        const size_t table_bytes = table_vals<T>(N) * sizeof(T);
         r.err = pick_warps(element_kernel<N, T, TX, OR, BD>, table_bytes, Ly::EWARP * sizeof(T), r.W, r.smem, r.per_sm);
         return r;
     }();
@@ -1205,7 +1207,6 @@ template <typename T, typename TX>
 cudaError_t launch_fused_warp(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y, cudaStream_t st,
                               int* launches) {
     const size_t cap = 220 * 1024;
-    const int ftot = sizeof(T) == 4 ? L.ft.total : 0;
     size_t max_tw = 0, max_ew = 0, max_tv = 0;
     for (int n = kMinN; n <= kMaxN; ++n) {
         if (buckets[n].count == 0) continue;
@@ -1213,7 +1214,7 @@ cudaError_t launch_fused_warp(const LevelView<T>& L, const BucketInfo* buckets, 
         DG_N_SWITCH(n, (tw = Layout<NN>::TWARP, ew = Layout<NN>::EWARP))
         max_tw = std::max(max_tw, tw);
         max_ew = std::max(max_ew, ew);
-        max_tv = std::max(max_tv, (size_t)(r4(ftot) + vol_vals(n)));
+        max_tv = std::max(max_tv, (size_t)table_vals<T>(n));
     }
     if (max_ew == 0) return cudaSuccess;
     int W = kFusedWarps;   // same CTA shape for every bucket; shrink until the largest degree fits
@@ -1253,7 +1254,6 @@ template <typename T, typename TX>
 cudaError_t launch_fused_cta(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y, cudaStream_t st,
                              int* launches) {
     const size_t cap = 220 * 1024;
-    const int ftot = sizeof(T) == 4 ? L.ft.total : 0;
     size_t smem_t = 0, smem_e = 0;
     FusedBuckets fb{};
     int ctas = 0;
@@ -1263,7 +1263,7 @@ cudaError_t launch_fused_cta(const LevelView<T>& L, const BucketInfo* buckets, c
         size_t tsh = 0, tw = 0, esh = 0, ew = 0;
         DG_N_SWITCH(n, (tsh = CtaLayout<NN>::TSHARED, tw = CtaLayout<NN>::TWARP, esh = CtaLayout<NN>::ESHARED,
                         ew = CtaLayout<NN>::EWARP))
-        const size_t tv = (size_t)(r4(ftot) + vol_vals(n));
+        const size_t tv = (size_t)table_vals<T>(n);
         smem_t = std::max(smem_t, (tv + tsh + kCtaWarps * tw) * sizeof(T));
         smem_e = std::max(smem_e, (tv + esh + kCtaWarps * ew) * sizeof(T));
         fb.n[fb.nb] = n;

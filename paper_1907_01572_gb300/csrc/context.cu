@@ -71,7 +71,6 @@ LevelView<double> level_view<double>(dg_ctx* c, int l) {
     v.sigma = L.sigma64;
     v.tab = c->tab64;
     v.ftab = c->ftab64;
-    v.ft = c->ft;
     v.ob_total = (long long)L.ob_count;
     v.oriented = L.oriented;
     v.chk = device_check_flag();
@@ -101,7 +100,6 @@ LevelView<float> level_view<float>(dg_ctx* c, int l) {
     v.sigma = L.sigma32;
     v.tab = c->tab32;
     v.ftab = c->ftab32;
-    v.ft = c->ft;
     v.ob_total = (long long)L.ob_count;
     v.oriented = L.oriented;
     v.chk = device_check_flag();
@@ -317,13 +315,13 @@ int smooth_t(dg_ctx* c, int l, const T* b, T* x, const dg_cheb_opts* o) {
     CK(smooth_init<T>(W.sm, b, W.Ap, W.r, W.p, n, c->red, st));
     c->launches += 1;
     const bool one = cg_step_fits<T>(n);
+    for (int k = 0; k < ne; ++k) {
+        if ((rc = solver_apply<T>(c, l, W.p, W.Ap))) return rc;
         if (one) {
             CK(cg_step_cluster<T>(W.sm, x, W.r, W.p, W.Ap, n, st));
             c->launches += 1;
             continue;
         }
-    for (int k = 0; k < ne; ++k) {
-        if ((rc = solver_apply<T>(c, l, W.p, W.Ap))) return rc;
         CK(cg_alpha_fused<T>(W.sm, W.p, W.Ap, n, c->red, st));
         CK(cg_update_fused<T>(W.sm, x, W.r, W.p, W.Ap, n, c->red, st));
         CK(cg_p_update<T>(W.sm, W.p, W.r, n, st));
@@ -1188,7 +1186,7 @@ int dg_ctx_create(const dg_mesh* mesh, const dg_disc_opts* opts, void* stream, d
     c->tab64 = c->arena.upload(tab, c->st);
     c->tab32 = c->arena.upload(tabf, c->st);
     std::vector<double> ftab;
-    build_face_tables(tab, ftab, c->ft);
+    build_face_tables(tab, ftab);
     std::vector<float> ftabf(ftab.begin(), ftab.end());
     c->ftab64 = c->arena.upload(ftab, c->st);
     c->ftab32 = c->arena.upload(ftabf, c->st);

@@ -142,16 +142,11 @@ void build_tables(std::vector<double>& tab) {
             }
 }
 
-void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab, FaceTabs& ft) {
+void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab) {
     ftab.clear();
     for (int n = kMinN; n <= kMaxN; ++n)
-        for (int q = kMinN; q <= kMaxN; ++q)
-            for (int pos = 0; pos < 3; ++pos) {
-                if (q < n) {
-                    ft.off[n - kMinN][q - kMinN][pos] = -1;
-                    continue;
-                }
-                ft.off[n - kMinN][q - kMinN][pos] = (int)ftab.size();   // even: pairs stay aligned
+        for (int q = n; q <= kMaxN; ++q)
+            for (int pos = 0; pos < 3; ++pos) {   // in the order of face_seg_off and face_tab_off
                 const double* Im = &tab[tab_m(TabIndex::Im, n, q, pos)];
                 const double* Dm = &tab[tab_m(TabIndex::Dm, n, q, pos)];
                 for (int k = 0; k < q * n; ++k) {
@@ -159,7 +154,6 @@ void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab
                     ftab.push_back(Dm[k]);
                 }
             }
-    ft.total = (int)ftab.size();
 }
 
 }  // namespace dg

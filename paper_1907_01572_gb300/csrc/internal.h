@@ -51,14 +51,15 @@ __host__ __device__ inline int tab_ci(int nH, int nh, int b) {
 
 void build_tables(std::vector<double>& tab);   // size TabIndex::Count * kTabStride
 
-// Compact mortar tables for the apply kernel's shared memory: for every side
-// degree n and mortar q >= n (q = max of both sides' n), sub-face pos 0..2,
-// the q x n matrices Im then Dm, packed without padding.
-struct FaceTabs {
-    int off[kNumN][kNumN][3];   // [n-2][q-2][pos] -> offset of the q*n (Im, Dm) pairs (even); -1 if q < n
-    int total;
-};
-void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab, FaceTabs& ft);
+// Compact mortar tables for the apply kernels' shared memory: one segment per
+// side n, holding for every mortar q >= n (q = max of both sides' n) and
+// sub-face pos 0..2 the q x n (Im, Dm) pairs, packed without padding.
+__host__ __device__ constexpr int face_seg_vals(int n) { return 6 * n * (kMaxN * (kMaxN + 1) / 2 - n * (n - 1) / 2); }
+__host__ __device__ constexpr int face_seg_off(int n) { return n <= kMinN ? 0 : face_seg_off(n - 1) + face_seg_vals(n - 1); }
+__host__ __device__ constexpr int face_tab_off(int n, int q, int pos) {   // inside n's segment (even)
+    return 2 * n * (3 * (q * (q - 1) / 2 - n * (n - 1) / 2) + pos * q);
+}
+void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab);
 
 // ---- mesh ----------------------------------------------------------------------
 struct Mortar {            // device record (32 bytes)
@@ -155,8 +156,7 @@ struct LevelView {         // passed by value to kernels
     const T* mg;           // 7 * n_mortar_pts: [wS, cA0, cA1, cA2, cB0, cB1, cB2] blocks per mortar
     const T* sigma;        // per mortar
     const T* tab;
-    const T* ftab;         // compact mortar tables (FaceTabs layout)
-    FaceTabs ft;
+    const T* ftab;         // compact mortar tables (face_seg_off, face_tab_off)
     long long ob_total;    // entries of Ob (bounds check)
     int oriented;          // some mortar of the level has a turned side B (Mortar::orient != 0)
     int bdiag;             // apply only the element diagonal blocks (the neighbour's trace taken as 0)
