@@ -602,7 +602,6 @@ struct Layout {
     // Element kernel: Y, A, G1, U (the input buffer, dead after the first
     // volume pass, holds the z-gradient); in the face phase A, G1 and U hold
     // the face scratch (flux factors and lift partial sums).
-    static constexpr bool UALIAS = true;
     static constexpr int EFACE = 4 * kQ * kQ + 3 * kQ * N;            // element kernel face scratch
     static constexpr int EWARP = r4(NR + (3 * NR > EFACE ? 3 * NR : EFACE));
 };
@@ -810,7 +809,6 @@ __device__ __forceinline__ void element_body(const LevelView<T>& L, const ElemDe
         const ElemDesc d = nd;
         const bool more = ei + stride < count;
         if (more) nd = bdesc[ei + stride];   // the next element's offsets, in flight during this one
-        const int e = d.e;
         const long long dofo = d.dofo, vo = d.vo;
         WarpSlots<T> ws;
         ws.load(L, d.s0, d.s1, lane);
@@ -871,22 +869,6 @@ __device__ __forceinline__ void element_body(const LevelView<T>& L, const ElemDe
         __syncwarp();
         vpass<N, 2, 1, false>(U, Y, sI, fr, lane);
         __syncwarp();
-        if (L.Ob != nullptr && L.Ob_off[e] + (long long)N3 * N3 > L.ob_total) {
-            if (lane == 0) atomicExch(L.chk, 1);
-        } else if (L.Ob != nullptr) {
-            // (coarse levels only; kept rolled so that its loads do not inflate
-            // the register count of the whole kernel)
-            const T* Oe = L.Ob + L.Ob_off[e];
-#pragma unroll 1
-            for (int k = lane; k < N3; k += 32) {
-                T s = 0;
-#pragma unroll 1
-                for (int j = 0; j < N3; ++j)   // u from the input vector when its buffer was reused
-                    s += Oe[(long long)j * N3 + k] * (Ly::UALIAS ? ld<T>(x + dofo + j) : U[sidx<N>(j)]);
-                Y[sidx<N>(k)] += s;
-            }
-            __syncwarp();
-        }
         for (int si = ws.s0; si < ws.s1; ++si) {
             const SlotRec<T> r = ws.get(si);
             const SlotInfo<T> s = unpack_rec(r);
@@ -896,7 +878,11 @@ __device__ __forceinline__ void element_body(const LevelView<T>& L, const ElemDe
             DG_Q_SWITCH(s.q, (lift_slot<N, Q, T, OR, BDM>(L, s, interior, r.sig, Y, sDL, sFT, F, mg, co, L.mt + 4 * s.goff,
                                                  lane)))
         }
-        for (int k = lane; k < N3; k += 32) __stcs(y + dofo + k, Y[sidx<N>(k)]);   // written once: evict first
+        if (L.Ob == nullptr) {
+            for (int k = lane; k < N3; k += 32) __stcs(y + dofo + k, Y[sidx<N>(k)]);   // written once: evict first
+        } else {   // y holds the Galerkin blocks' part (galerkin_apply_kernel)
+            for (int k = lane; k < N3; k += 32) y[dofo + k] += Y[sidx<N>(k)];
+        }
         __syncwarp();
     }
 }
@@ -1057,16 +1043,6 @@ __device__ __forceinline__ void element_body_cta(const LevelView<T>& L, int e, c
     __syncthreads();
     wpass<N, 2, true, false>(B, Y, sI, tid, nt);
     __syncthreads();
-    if (L.Ob != nullptr && L.Ob_off[e] + (long long)N3 * N3 > L.ob_total) {
-        if (tid == 0) atomicExch(L.chk, 1);
-    } else if (L.Ob != nullptr) {
-        const T* Oe = L.Ob + L.Ob_off[e];
-        for (int k = tid; k < N3; k += nt) {
-            T sacc = 0;
-            for (int j = 0; j < N3; ++j) sacc += Oe[(long long)j * N3 + k] * U[sidx<N>(j)];
-            Y[sidx<N>(k)] += sacc;
-        }
-    }
     for (int k = lane; k < NR; k += 32) Yw[k] = 0;
     __syncwarp();
     const int s0 = L.slot_off[e], s1 = L.slot_off[e + 1];
@@ -1084,6 +1060,7 @@ __device__ __forceinline__ void element_body_cta(const LevelView<T>& L, int e, c
         const int s = sidx<N>(k);
         T acc = Y[s];
         for (int w = 0; w < nw; ++w) acc += base[Ly::ESHARED + w * Ly::EWARP + s];
+        if (L.Ob != nullptr) acc += y[dofo + k];   // the Galerkin blocks' part (galerkin_apply_kernel)
         __stcs(y + dofo + k, acc);
     }
 }
@@ -1100,6 +1077,55 @@ __global__ void element_cta(LevelView<T> L, FusedBuckets fb, const TX* __restric
     const int b = fused_bucket(fb);
     const int e = fb.elems[b][blockIdx.x - fb.cta_start[b]];
     DG_BODY_SWITCH(fb.n[b], (element_body_cta<NN, T, TX>(L, e, x, y)))
+}
+
+// ---- Galerkin blocks of the zeroth-order term (coarse levels) ----------------------
+// y_e = O_e x_e with the dense n^3 x n^3 block O_e (column-major), ahead of the
+// element kernels, which add their part to y.  A block of 256 threads takes 32
+// rows of one element; its warps split the columns and are summed in warp
+// order.  Bounded by reading the blocks (470 KB per element at n = 7 in FP32),
+// which rows spread over the whole chip do at memory speed: inside the element
+// kernel, one CTA read its element's block alone (27 elements, n <= 7, FP32: an
+// apply with the blocks took 56 us, 31 more than without; now 21.6 us, 4.6 more).
+constexpr int kObRows = 32, kObWarps = 8;
+
+template <typename T, typename TX>
+__global__ void __launch_bounds__(kObWarps * 32)
+    galerkin_apply_kernel(LevelView<T> L, const TX* __restrict__ x, T* __restrict__ y) {
+    __shared__ T xs[kMaxN * kMaxN * kMaxN], part[kObWarps][kObRows];
+    const int e = blockIdx.x, n = L.p[e] + 1, n3 = n * n * n, r0 = blockIdx.y * kObRows;
+    if (r0 >= n3) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long off = L.Ob_off[e], dofo = L.dof_off[e];
+    const bool ok = off >= 0 && off + (long long)n3 * n3 <= L.ob_total;
+    if (!ok && threadIdx.x == 0) atomicExch(L.chk, 1);
+    for (int k = threadIdx.x; k < n3; k += blockDim.x) xs[k] = ld<T>(x + dofo + k);
+    __syncthreads();
+    const int row = r0 + lane;
+    T s = 0;
+    if (ok && row < n3) {
+        const T* O = L.Ob + off + row;
+#pragma unroll 8
+        for (int j = warp; j < n3; j += kObWarps) s += O[(long long)j * n3] * xs[j];
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && row < n3) {
+        T t = 0;
+        for (int w = 0; w < kObWarps; ++w) t += part[w][lane];
+        y[dofo + row] = t;
+    }
+}
+
+template <typename T, typename TX>
+cudaError_t launch_galerkin_apply(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
+                                  cudaStream_t st, int* launches) {
+    int n = kMaxN;
+    while (n > kMinN && buckets[n].count == 0) --n;
+    const dim3 grid(L.n_elems, (n * n * n + kObRows - 1) / kObRows);
+    galerkin_apply_kernel<T, TX><<<grid, kObWarps * 32, 0, st>>>(L, x, y);
+    if (launches) ++*launches;
+    return cudaGetLastError();
 }
 
 // Launch shape of a per-bucket kernel, found once per template instance.  The
@@ -1295,7 +1321,7 @@ cudaError_t launch_fused_cta(const LevelView<T>& L, const BucketInfo* buckets, c
 }  // namespace apply_detail
 
 template <typename T, typename TX>
-cudaError_t launch_path(int path, const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
+cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
                         cudaStream_t st, int* launches, const ApplyStreams* as) {
     if (path == 0) return apply_detail::launch_fused_cta<T, TX>(L, buckets, x, y, st, launches);
     if (path == 1) return apply_detail::launch_fused_warp<T, TX>(L, buckets, x, y, st, launches);
@@ -1340,6 +1366,16 @@ cudaError_t launch_path(int path, const LevelView<T>& L, const BucketInfo* bucke
         }
     }
     return cudaSuccess;
+}
+
+template <typename T, typename TX>
+cudaError_t launch_path(int path, const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
+                        cudaStream_t st, int* launches, const ApplyStreams* as) {
+    if (L.Ob != nullptr) {
+        const cudaError_t err = apply_detail::launch_galerkin_apply<T, TX>(L, buckets, x, y, st, launches);
+        if (err != cudaSuccess) return err;
+    }
+    return launch_kernels<T, TX>(path, L, buckets, x, y, st, launches, as);
 }
 
 // Launch plan of a level: 0 one CTA per element, 1 one warp per element in a

@@ -1,7 +1,9 @@
-"""The CG step of the smoother's eigenvalue estimate: one cluster, or three
-launches on longer vectors."""
+"""Kernels that carry the small levels: the CG step of the smoother's eigenvalue
+estimate (one cluster, or three launches on longer vectors) and the product
+with the Galerkin blocks of the zeroth-order term."""
 import math
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -53,3 +55,35 @@ def test_cg_step_and_estimate(desc):
     # six CG steps amplify the rounding of the dot products (n eps) by at most a few hundred
     assert abs(got_lam - lam) <= 1e-11 * lam
     assert float((x - want).norm()) <= 1e-11 * float(want.norm())
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 6, 8])
+def test_galerkin_blocks_on_the_coarse_level(p):
+    """O^H x = (I^T O^h I) x, with O^h from the finest level's quadrature."""
+    ctx = dgell.Context(single(p, level=1, warp=(0.03, (1, 2, 1))))
+    assert ctx.n_levels == 2
+    nf, nc = ctx.level_info(1)["n_dofs"], ctx.level_info(0)["n_dofs"]
+    g = torch.Generator(device="cuda").manual_seed(p)
+    x = torch.randn(nc, dtype=torch.float64, device="cuda", generator=g)
+    coef = 1.0 + torch.rand(ctx.level_info(1)["n_vol_qp"], dtype=torch.float64, device="cuda", generator=g)
+    xf = torch.zeros(nf, dtype=torch.float64, device="cuda")
+    ctx.transfer(0, 0, x, xf)
+
+    def both(z):
+        ctx.set_zeroth_order(coef if z else None)
+        return [ctx.apply(v, torch.empty_like(v), level=l) for v, l in ((x, 0), (xf, 1))]
+
+    (c1, f1), (c0, f0) = both(True), both(False)
+    want = torch.empty_like(x)
+    ctx.transfer(0, 1, f1 - f0, want)
+    # both sides are differences of applies: their rounding is eps times the apply's size
+    size = float(c1.norm()) + float(f1.norm())
+    assert float((c1 - c0 - want).norm()) <= 1e-13 * size
+    ctx.set_zeroth_order(coef)
+    y32 = torch.empty(nc, device="cuda")
+    ctx.apply(x.float(), y32, level=0)
+    ctx.set_zeroth_order(None)
+    n32 = torch.empty(nc, device="cuda")
+    ctx.apply(x.float(), n32, level=0)
+    assert float((y32.double() - n32.double() - want).norm()) <= 1e-6 * size
+    assert np.isfinite(size)
