@@ -83,9 +83,10 @@ struct LevelDev {
     double* denseL = nullptr;         // its SIPG (Laplacian) part, built once; + Galerkin blocks -> dense64
     long long dense_version = -1;     // op_version the dense operator was built for
     int plan[3] = {-1, -1, -1};       // tuned apply launch plan per precision (FP64, FP32, BF16 operands)
-    // Galerkin structure of a coarse level: finest descendants and their reference maps
-    int *g_desc_off = nullptr, *g_desc = nullptr;
-    double* g_map = nullptr;
+    // zeroth-order term of a coarse level: its coefficient at (2p + 1)^3 GL points per element (newton.cu)
+    long long* g_off = nullptr;
+    double* g_coef = nullptr;
+    size_t g_count = 0;
     size_t ob_count = 0;
     // transfer to the next finer level (this level is the coarse side)
     int *child_off = nullptr, *child_id = nullptr, *fine_parent = nullptr;
@@ -129,6 +130,7 @@ struct dg_ctx {
     bool nl_has_F = false;
     double* nw[4] = {};             // Newton work vectors (double, finest): R, du, Lu, S
     bool galerkin_ready = false;
+    double* gal_tab = nullptr;      // GalerkinTab (newton.h)
     // CUDA graph of the V-cycle used inside dg_solve (captured once, replayed)
     cudaGraphExec_t vgraph = nullptr;
     int vgraph_prec = -1;

@@ -29,51 +29,35 @@ extern "C" int dgi_set_error(int code, const char* msg);
 
 namespace {
 
-// Finest descendants of every coarse element and the affine maps from their
-// reference coordinates to the ancestor's (xi_H = s xi_f + o per axis).
+// Coefficient and block buffers of the zeroth-order term on the coarse levels.
 int ensure_galerkin_structure(dg_ctx* c) {
     if (c->galerkin_ready) return DG_OK;
     const int Lt = (int)c->lv.size() - 1;
-    const LevelHost& fin = c->lv[Lt].h;
-    const int nf = fin.n_elems();
-    std::vector<int> anc(nf);
-    for (int f = 0; f < nf; ++f) anc[f] = f;
+    if (Lt > 0) {
+        std::vector<double> tab;
+        build_galerkin_tables(tab);
+        c->gal_tab = c->arena.upload(tab, c->st);
+        CK2(cudaStreamSynchronize(c->st));   // tab goes out of scope
+    }
     for (int l = Lt - 1; l >= 0; --l) {
         LevelDev& L = c->lv[l];
         const LevelHost& h = L.h;
-        for (int f = 0; f < nf; ++f) anc[f] = h.fine_parent[anc[f]];
         const int nc = h.n_elems();
-        std::vector<int> cnt(nc + 1, 0);
-        for (int f = 0; f < nf; ++f) cnt[anc[f] + 1]++;
-        for (int H = 0; H < nc; ++H) cnt[H + 1] += cnt[H];
-        std::vector<int> desc(nf), fill(cnt.begin(), cnt.end() - 1);
-        std::vector<double> map(6 * (size_t)nf);
-        for (int f = 0; f < nf; ++f) {
-            const int H = anc[f];
-            const int slot = fill[H]++;
-            desc[slot] = f;
-            const int* lf = &fin.leaves[4 * f];
-            const int* lH = &h.leaves[4 * H];
-            const int D = lf[0] - lH[0];
-            const double s = std::ldexp(1.0, -D);
-            for (int d = 0; d < 3; ++d) {
-                map[6 * (size_t)slot + 2 * d] = s;
-                map[6 * (size_t)slot + 2 * d + 1] = (2.0 * lf[1 + d] + 1.0) * s - 2.0 * lH[1 + d] - 1.0;
-            }
-        }
-        std::vector<long long> ob_off(nc + 1, 0);
+        std::vector<long long> ob_off(nc + 1, 0), g_off(nc + 1, 0);
         for (int H = 0; H < nc; ++H) {
-            const long long n3 = (long long)(h.p[H] + 1) * (h.p[H] + 1) * (h.p[H] + 1);
+            const long long n = h.p[H] + 1, n3 = n * n * n, m = 2 * n - 1;
             ob_off[H + 1] = ob_off[H] + n3 * n3;
+            g_off[H + 1] = g_off[H] + m * m * m;
         }
-        L.g_desc_off = c->arena.upload(cnt, c->st);
-        L.g_desc = c->arena.upload(desc, c->st);
-        L.g_map = c->arena.upload(map, c->st);
+        L.g_off = c->arena.upload(g_off, c->st);
         L.Ob_off = c->arena.upload(ob_off, c->st);
         L.ob_count = (size_t)ob_off.back();
+        L.g_count = (size_t)g_off.back();
+        L.g_coef = c->arena.alloc<double>(L.g_count);
         L.Ob64 = c->arena.alloc<double>(L.ob_count);
         L.Ob32 = c->arena.alloc<float>(L.ob_count);
         if (c->arena.failed) return dgi_set_error(DG_ERR_OOM, "device allocation failed (Galerkin blocks)");
+        CK2(cudaStreamSynchronize(c->st));   // the offsets go out of scope
     }
     LevelDev& F = c->lv[Lt];
     const size_t nv = (size_t)F.h.vqp_off.back();
@@ -86,28 +70,35 @@ int ensure_galerkin_structure(dg_ctx* c) {
     return DG_OK;
 }
 
-// Coarse-level Galerkin blocks from the finest-level c0 (already in F.c0_64); activates the term.
+// Coarse-level Galerkin blocks from the finest-level c0 (already in F.c0_64), level by level downwards;
+// activates the term.
 int build_galerkin(dg_ctx* c) {
     const int Lt = (int)c->lv.size() - 1;
     LevelDev& F = c->lv[Lt];
-    for (int l = 0; l < Lt; ++l) {
-        LevelDev& L = c->lv[l];
+    for (int l = Lt - 1; l >= 0; --l) {
+        LevelDev &L = c->lv[l], &f = c->lv[l + 1];
+        const bool top = l + 1 == Lt;
         GalerkinArgs g{};
         g.n_coarse = L.h.n_elems();
         g.pH = L.p;
+        g.pf = f.p;
+        g.fine_is_finest = top;
+        g.child_off = L.child_off;
+        g.child_id = L.child_id;
+        g.child_bits = L.child_bits;
+        g.off_f = top ? f.vqp_off : f.g_off;
+        g.off = L.g_off;
         g.Ob_off = L.Ob_off;
-        g.desc_off = L.g_desc_off;
-        g.desc = L.g_desc;
-        g.map = L.g_map;
-        g.pf = F.p;
-        g.vqp_off_f = F.vqp_off;
-        g.tab = c->tab64;
+        g.tab = c->gal_tab;
+        g.n_coef_f = top ? f.h.vqp_off.back() : (long long)f.g_count;
+        g.n_coef = (long long)L.g_count;
         g.ob_total = (long long)L.ob_count;
-        g.n_vqp_f = F.h.vqp_off.back();
-        g.n_desc = F.h.n_elems();
         g.chk = device_check_flag();
-        CK2(launch_galerkin(g, F.c0_64, L.Ob64, L.Ob32, c->st));
-        c->launches += 1;
+        int max_n = kMinN;
+        for (int n = kMinN; n <= kMaxN; ++n)
+            if (L.buckets[n].count > 0) max_n = n;
+        CK2(launch_galerkin(g, max_n, top ? f.c0_64 : f.g_coef, L.g_coef, L.Ob64, L.Ob32, c->st));
+        c->launches += 2;
         ++c->op_version;
         if (!L.z_active) ++c->epoch;
         L.z_active = true;

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "newton.h"
 
 namespace dg {
 namespace {
@@ -154,6 +155,26 @@ void build_face_tables(const std::vector<double>& tab, std::vector<double>& ftab
                     ftab.push_back(Dm[k]);
                 }
             }
+}
+
+void build_galerkin_tables(std::vector<double>& tab) {
+    tab.assign((size_t)GalerkinTab::Count * GalerkinTab::Stride, 0.0);
+    std::vector<double> x[kGalM + 1], w;
+    for (int q = 1; q <= kGalM; ++q) gl(q, x[q], w);
+    for (int n = kMinN; n <= kMaxN; ++n) {
+        const int m = 2 * n - 1;
+        for (int q = kMinN; q <= kGalM; ++q)
+            for (int b = 0; b < 3; ++b)
+                for (int k = 0; k < m; ++k)
+                    for (int j = 0; j < q; ++j) {
+                        const double t = b == 2 ? x[q][j] : 0.5 * (x[q][j] + 2.0 * b - 1.0);
+                        tab[GalerkinTab::w(n, q, b) + k * kGalM + j] = lag(x[m], k, t);
+                    }
+        std::vector<double> xl, wl;
+        lgl(n, xl, wl);
+        for (int k = 0; k < m; ++k)
+            for (int a = 0; a < n; ++a) tab[GalerkinTab::e(n) + k * kGalM + a] = lag(xl, a, x[m][k]);
+    }
 }
 
 }  // namespace dg

@@ -5,10 +5,17 @@
 //   coefficient c0 = w det J f folded into the apply kernel.
 // * Coarse levels: the Galerkin form O^H = (I_h^H)^T O^h I_h^H.  Because the
 //   prolongation interpolates exactly (coarse spaces are nested in the fine
-//   ones), O^H_ab = sum over the finest descendants' GL points of
-//   c0 psi^H_a psi^H_b, with psi^H evaluated at those points.  The kernel sums
-//   this per descendant in sum-factorised form (first over the z points for
-//   every pair (c, c'), then over x and y per matrix entry).
+//   ones), O^H_ab = sum over the finest descendants' GL points x_q of
+//   c0_q phi(x_q) with phi = psi^H_a psi^H_b, a polynomial of degree 2p per
+//   direction, which its values at the m = 2p + 1 GL points y_k of the coarse
+//   element determine: phi(x_q) = sum_k L_k(x_q) phi(y_k).  So the coarse
+//   coefficient c_k = sum_q c0_q L_k(x_q) carries the whole term, and (spaces
+//   nested level by level) it follows from the next finer level's coefficient
+//   by one transposed interpolation per child.  The dense block is then
+//   O^H_ab = sum_k c_k psi_a(y_k) psi_b(y_k), summed direction by direction over
+//   the pairs (c, c'), (b, b'), (a, a') with c <= c' and so on.  Work per
+//   element at n = 7: 0.3 M multiply-adds and 0.1 M per child (summing every
+//   entry over every finest point: 6.6 M per finest descendant).
 // * Puncture: 1/alpha = sum_I m_I / (2 r_I); A_ij = sum_I 3/(2 r_I^2)
 //   [P_i n_j + P_j n_i - (delta_ij - n_i n_j) P.n] + 3/r_I^3 [n_i w_j + n_j w_i],
 //   w = S_I x n (the spin term of eq. Two_Punctures_Aij, its symmetrisation
@@ -22,13 +29,6 @@
 
 namespace dg {
 namespace {
-
-__device__ inline double lagv(const double* x, int n, int a, double t) {
-    double v = 1.0;
-    for (int m = 0; m < n; ++m)
-        if (m != a) v *= (t - x[m]) / (x[a] - x[m]);
-    return v;
-}
 
 __global__ void puncture_kernel(const double* vxyz, long long n, PunctureDev P, double* alpha, double* beta) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -151,74 +151,119 @@ __global__ void sub_kernel(const double* Lu, const double* S, const double* F, d
         R[i] = Lu[i] - S[i] - (F ? F[i] : 0.0);
 }
 
-// O_H for every coarse element H of one level (block per H, loop over its finest descendants).
-__global__ void galerkin_kernel(GalerkinArgs g, const double* c0, double* O64, float* O32) {
+// out (= or +=) sum_j W[k][j] in[.. j ..]: one direction of a transposed interpolation, of a cube with
+// dims (d0, d1, d2) to m points along `dir`.
+__device__ void interp_pass(const double* in, double* out, const double* W, int dir, int d0, int d1, int d2, int m,
+                            bool add) {
+    const int q = dir == 0 ? d0 : (dir == 1 ? d1 : d2);
+    const int e0 = dir == 0 ? m : d0, e1 = dir == 1 ? m : d1, e2 = dir == 2 ? m : d2;
+    const int si = dir == 0 ? 1 : (dir == 1 ? d0 : d0 * d1);
+    for (int idx = threadIdx.x; idx < e0 * e1 * e2; idx += blockDim.x) {
+        const int a = idx % e0, b = (idx / e0) % e1, c = idx / (e0 * e1);
+        const int k = dir == 0 ? a : (dir == 1 ? b : c);
+        const double* v = in + (dir == 0 ? 0 : a) + d0 * ((dir == 1 ? 0 : b) + d1 * (dir == 2 ? 0 : c));
+        const double* w = W + k * kGalM;
+        double s = 0.0;
+        for (int j = 0; j < q; ++j) s += w[j] * v[j * si];
+        out[idx] = add ? out[idx] + s : s;
+    }
+}
+
+// Coefficients of one coarse level (block per element, its children in turn).
+__global__ void galerkin_coef_kernel(GalerkinArgs g, const double* __restrict__ cf, double* __restrict__ coef) {
+    extern __shared__ double gal_smem[];
+    constexpr int M3 = kGalM * kGalM * kGalM;
+    double *b0 = gal_smem, *b1 = b0 + M3, *acc = b1 + M3;
     const int H = blockIdx.x;
-    if (H >= g.n_coarse) return;
-    const int nH = g.pH[H] + 1, nH2 = nH * nH, nH3 = nH2 * nH;
-    const long long nent = (long long)nH3 * nH3;
-    if (nH < kMinN || nH > kMaxN || g.Ob_off[H] < 0 || g.Ob_off[H] + nent > g.ob_total) {
+    const int n = g.pH[H] + 1, m = 2 * n - 1, m3 = m * m * m;
+    const long long off = g.off[H];
+    if (n < kMinN || n > kMaxN || off < 0 || off + m3 > g.n_coef) {
         if (threadIdx.x == 0) atomicExch(g.chk, 3);
         return;
     }
-    double* Oe = O64 + g.Ob_off[H];
-    __shared__ double E[3][kMaxN * kMaxN];          // E_d[i][a]
-    __shared__ double xlH[kMaxN], xgq[kMaxN];
-    extern __shared__ double dyn[];
-    double* T1 = dyn;                               // T1[(c, c')][i][j], n_H^2 q^2 <= 9^4
-    double* cq = dyn + kMaxN * kMaxN * kMaxN * kMaxN;   // c0 at the descendant's GL points
-    for (long long k = threadIdx.x; k < nent; k += blockDim.x) Oe[k] = 0.0;
-    if (threadIdx.x < nH) xlH[threadIdx.x] = g.tab[tab_n(TabIndex::LGLx, nH) + threadIdx.x];
-    __syncthreads();
-    for (int di = g.desc_off[H]; di < g.desc_off[H + 1]; ++di) {
-        if (di < 0 || di >= g.n_desc) {
+    for (int k = threadIdx.x; k < m3; k += blockDim.x) acc[k] = 0.0;
+    for (int ci = g.child_off[H]; ci < g.child_off[H + 1]; ++ci) {
+        const int f = g.child_id[ci], bits = g.child_bits[ci];
+        const int nf = g.pf[f] + 1, q = g.fine_is_finest ? nf : 2 * nf - 1, q3 = q * q * q;
+        const long long of = g.off_f[f];
+        if (nf < kMinN || nf > kMaxN || of < 0 || of + q3 > g.n_coef_f) {
             if (threadIdx.x == 0) atomicExch(g.chk, 4);
             break;
         }
-        const int f = g.desc[di];
-        const int q = g.pf[f] + 1, q2 = q * q, q3 = q2 * q;
-        const long long vo = g.vqp_off_f[f];
-        if (q < kMinN || q > kMaxN || vo < 0 || vo + q3 > g.n_vqp_f) {
-            if (threadIdx.x == 0) atomicExch(g.chk, 5);
-            break;
-        }
-        if (threadIdx.x < q) xgq[threadIdx.x] = g.tab[tab_n(TabIndex::GLx, q) + threadIdx.x];
-        for (int k = threadIdx.x; k < q3; k += blockDim.x) cq[k] = c0[vo + k];
+        for (int k = threadIdx.x; k < q3; k += blockDim.x) b0[k] = cf[of + k];
         __syncthreads();
-        const double* so = g.map + 6 * (long long)di;   // scale and offset per axis
-        for (int k = threadIdx.x; k < 3 * q * nH; k += blockDim.x) {
-            const int dd = k / (q * nH), r = k % (q * nH), i = r / nH, a = r % nH;
-            E[dd][i * nH + a] = lagv(xlH, nH, a, so[2 * dd] * xgq[i] + so[2 * dd + 1]);
-        }
+        const double* W[3];
+        for (int d = 0; d < 3; ++d) W[d] = g.tab + GalerkinTab::w(n, q, bits == 0xFF ? 2 : (bits >> d) & 1);
+        interp_pass(b0, b1, W[0], 0, q, q, q, m, false);
         __syncthreads();
-        // T1[(c, c')][i][j] = sum_k c0[i, j, k] Ez[k, c] Ez[k, c']
-        for (int k = threadIdx.x; k < nH2 * q2; k += blockDim.x) {
-            const int cc = k / q2, ij = k % q2;
-            const int c = cc / nH, c2 = cc % nH;
-            double s = 0.0;
-            for (int kk = 0; kk < q; ++kk) s += cq[ij + q2 * kk] * E[2][kk * nH + c] * E[2][kk * nH + c2];
-            T1[k] = s;
-        }
+        interp_pass(b1, b0, W[1], 1, m, q, q, m, false);
         __syncthreads();
-        // O[(a, b, c), (a', b', c')] += sum_{i, j} Ex[i,a] Ex[i,a'] Ey[j,b] Ey[j,b'] T1[(c,c')][i][j]
-        for (long long k = threadIdx.x; k < nent; k += blockDim.x) {
-            const int al = (int)(k / nH3), be = (int)(k % nH3);
-            const int a = al % nH, b = (al / nH) % nH, c = al / nH2;
-            const int a2 = be % nH, b2 = (be / nH) % nH, c2 = be / nH2;
-            const double* t = T1 + (c * nH + c2) * q2;
-            double s = 0.0;
-            for (int j = 0; j < q; ++j) {
-                const double ey = E[1][j * nH + b] * E[1][j * nH + b2];
-                double sx = 0.0;
-                for (int i = 0; i < q; ++i) sx += E[0][i * nH + a] * E[0][i * nH + a2] * t[i + q * j];
-                s += ey * sx;
-            }
-            Oe[k] += s;
-        }
+        interp_pass(b0, acc, W[2], 2, m, m, q, m, true);
         __syncthreads();
     }
-    float* Of = O32 + g.Ob_off[H];
-    for (long long k = threadIdx.x; k < nent; k += blockDim.x) Of[k] = (float)Oe[k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < m3; k += blockDim.x) coef[off + k] = acc[k];
+}
+
+// Entries of one element's block with z indices (c, c') or (c', c): a CTA per pair.
+__global__ void galerkin_block_kernel(GalerkinArgs g, const double* __restrict__ coef, double* __restrict__ O64,
+                                      float* __restrict__ O32) {
+    constexpr int NP = kMaxN * (kMaxN + 1) / 2;
+    __shared__ double E[kGalM][kMaxN], ez[kGalM], T1[kGalM * kGalM], T2[NP][kGalM], S[NP][NP];
+    __shared__ unsigned char pa[NP], pb[NP];
+    const int H = blockIdx.x, n = g.pH[H] + 1, n3 = n * n * n, m = 2 * n - 1, np = n * (n + 1) / 2;
+    if ((int)blockIdx.y >= np) return;
+    const long long off = g.off[H], oo = g.Ob_off[H];
+    if (n < kMinN || n > kMaxN || off < 0 || off + m * m * m > g.n_coef || oo < 0 || oo + (long long)n3 * n3 > g.ob_total) {
+        if (threadIdx.x == 0) atomicExch(g.chk, 5);
+        return;
+    }
+    for (int k = threadIdx.x; k < m * n; k += blockDim.x) E[k / n][k % n] = g.tab[GalerkinTab::e(n) + (k / n) * kGalM + k % n];
+    for (int k = threadIdx.x; k < n * n; k += blockDim.x) {
+        const int a = k % n, b = k / n;
+        if (a <= b) {
+            pa[b * (b + 1) / 2 + a] = a;
+            pb[b * (b + 1) / 2 + a] = b;
+        }
+    }
+    __syncthreads();
+    const int c = pa[blockIdx.y], c2 = pb[blockIdx.y];
+    if (threadIdx.x < m) ez[threadIdx.x] = E[threadIdx.x][c] * E[threadIdx.x][c2];
+    __syncthreads();
+    for (int ij = threadIdx.x; ij < m * m; ij += blockDim.x) {
+        double s = 0.0;
+        for (int k = 0; k < m; ++k) s += coef[off + ij + m * m * k] * ez[k];
+        T1[ij] = s;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < np * m; k += blockDim.x) {
+        const int i = k % m, b = k / m;
+        double s = 0.0;
+        for (int j = 0; j < m; ++j) s += T1[i + m * j] * (E[j][pa[b]] * E[j][pb[b]]);
+        T2[b][i] = s;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < np * np; k += blockDim.x) {
+        const int a = k % np, b = k / np;
+        double s = 0.0;
+        for (int i = 0; i < m; ++i) s += T2[b][i] * (E[i][pa[a]] * E[i][pb[a]]);
+        S[b][a] = s;
+    }
+    __syncthreads();
+    const int n2 = n * n;
+    for (int k = threadIdx.x; k < n2 * n2; k += blockDim.x) {   // rows (a', b') fastest: runs of n^2 values
+        const int r = k % n2, l = k / n2;
+        const int a2 = r % n, b2 = r / n, a = l % n, b = l / n;
+        const int ia = a < a2 ? a2 * (a2 + 1) / 2 + a : a * (a + 1) / 2 + a2;
+        const int ib = b < b2 ? b2 * (b2 + 1) / 2 + b : b * (b + 1) / 2 + b2;
+        const double v = S[ib][ia];
+        const long long p0 = oo + (long long)(l + n2 * c) * n3 + r + n2 * c2;
+        const long long p1 = oo + (long long)(l + n2 * c2) * n3 + r + n2 * c;
+        O64[p0] = v;
+        O64[p1] = v;
+        O32[p0] = (float)v;
+        O32[p1] = (float)v;
+    }
 }
 
 inline int grid_for(long long n) {
@@ -244,12 +289,14 @@ cudaError_t launch_sub(const double* Lu, const double* S, const double* F, doubl
     return cudaGetLastError();
 }
 
-cudaError_t launch_galerkin(const GalerkinArgs& g, const double* c0, double* O64, float* O32, cudaStream_t st) {
-    const size_t smem = sizeof(double) * (kMaxN * kMaxN * kMaxN * kMaxN + kMaxN * kMaxN * kMaxN);
+cudaError_t launch_galerkin(const GalerkinArgs& g, int max_n, const double* coef_f, double* coef, double* O64,
+                            float* O32, cudaStream_t st) {
+    const size_t smem = sizeof(double) * 3 * kGalM * kGalM * kGalM;
     static const cudaError_t attr =   // once per process, thread-safe initialisation
-        cudaFuncSetAttribute(galerkin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(galerkin_coef_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess) return attr;
-    galerkin_kernel<<<g.n_coarse, 256, smem, st>>>(g, c0, O64, O32);
+    galerkin_coef_kernel<<<g.n_coarse, 512, smem, st>>>(g, coef_f, coef);
+    galerkin_block_kernel<<<dim3(g.n_coarse, max_n * (max_n + 1) / 2), 128, 0, st>>>(g, coef, O64, O32);
     return cudaGetLastError();
 }
 

@@ -3,7 +3,6 @@ estimate (one cluster, or three launches on longer vectors) and the product
 with the Galerkin blocks of the zeroth-order term."""
 import math
 
-import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -57,33 +56,41 @@ def test_cg_step_and_estimate(desc):
     assert float((x - want).norm()) <= 1e-11 * float(want.norm())
 
 
-@pytest.mark.parametrize("p", [1, 2, 3, 6, 8])
-def test_galerkin_blocks_on_the_coarse_level(p):
+def _curved(p):
+    return single(p, level=1, warp=(0.03, (1, 2, 1)))
+
+
+# every remainder of the 32 rows a block takes; elements carried over between levels and mixed degrees on
+# three levels; turned blocks
+@pytest.mark.parametrize("desc", [_curved(1), _curved(2), _curved(3), _curved(6), _curved(8),
+                                  inputs.sweep_mesh(level=1, seed=3, pmin=1, pmax=8),
+                                  inputs.block_pair_mesh(rot=5, level=2, seed=1)],
+                         ids=["p1", "p2", "p3", "p6", "p8", "hp", "blocks"])
+def test_galerkin_blocks_on_the_coarse_levels(desc):
     """O^H x = (I^T O^h I) x, with O^h from the finest level's quadrature."""
-    ctx = dgell.Context(single(p, level=1, warp=(0.03, (1, 2, 1))))
-    assert ctx.n_levels == 2
-    nf, nc = ctx.level_info(1)["n_dofs"], ctx.level_info(0)["n_dofs"]
-    g = torch.Generator(device="cuda").manual_seed(p)
-    x = torch.randn(nc, dtype=torch.float64, device="cuda", generator=g)
-    coef = 1.0 + torch.rand(ctx.level_info(1)["n_vol_qp"], dtype=torch.float64, device="cuda", generator=g)
-    xf = torch.zeros(nf, dtype=torch.float64, device="cuda")
-    ctx.transfer(0, 0, x, xf)
+    ctx = dgell.Context(desc)
+    Lt = ctx.n_levels - 1
+    assert Lt >= 1
+    n = [ctx.level_info(l)["n_dofs"] for l in range(Lt + 1)]
+    g = torch.Generator(device="cuda").manual_seed(n[0])
+    coef = 1.0 + torch.rand(ctx.level_info()["n_vol_qp"], dtype=torch.float64, device="cuda", generator=g)
+    for low in range(Lt):
+        x = torch.randn(n[low], dtype=torch.float64, device="cuda", generator=g)
+        xf = x
+        for l in range(low, Lt):
+            up = torch.zeros(n[l + 1], dtype=torch.float64, device="cuda")
+            xf = ctx.transfer(l, 0, xf, up)
 
-    def both(z):
-        ctx.set_zeroth_order(coef if z else None)
-        return [ctx.apply(v, torch.empty_like(v), level=l) for v, l in ((x, 0), (xf, 1))]
+        def both(z):
+            ctx.set_zeroth_order(coef if z else None)
+            lowp = ctx.apply(x.float(), torch.empty(n[low], device="cuda"), level=low)
+            return [ctx.apply(x, torch.empty_like(x), level=low), ctx.apply(xf, torch.empty_like(xf)), lowp.double()]
 
-    (c1, f1), (c0, f0) = both(True), both(False)
-    want = torch.empty_like(x)
-    ctx.transfer(0, 1, f1 - f0, want)
-    # both sides are differences of applies: their rounding is eps times the apply's size
-    size = float(c1.norm()) + float(f1.norm())
-    assert float((c1 - c0 - want).norm()) <= 1e-13 * size
-    ctx.set_zeroth_order(coef)
-    y32 = torch.empty(nc, device="cuda")
-    ctx.apply(x.float(), y32, level=0)
-    ctx.set_zeroth_order(None)
-    n32 = torch.empty(nc, device="cuda")
-    ctx.apply(x.float(), n32, level=0)
-    assert float((y32.double() - n32.double() - want).norm()) <= 1e-6 * size
-    assert np.isfinite(size)
+        (c1, f1, s1), (c0, f0, s0) = both(True), both(False)
+        want = f1 - f0
+        for l in range(Lt - 1, low - 1, -1):
+            want = ctx.transfer(l, 1, want, torch.empty(n[l], dtype=torch.float64, device="cuda"))
+        # both sides are differences of applies: their rounding is that of the applies
+        size = float(c1.norm()) + float(f1.norm())
+        assert float((c1 - c0 - want).norm()) <= 1e-13 * size
+        assert float((s1 - s0 - want).norm()) <= 1e-6 * size
