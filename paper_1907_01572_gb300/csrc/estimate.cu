@@ -29,48 +29,187 @@ namespace {
 
 constexpr int kEstThreads = 768;   // >= kMaxN^3 = 729
 constexpr int kNV = kMaxN * kMaxN * kMaxN;
+constexpr int kEstMaxSlots = 24;   // four mortars on each of six faces
 
-// Derivative (d0, d1, d2) of the nodal field F (n^3 values, x fastest) at GL
-// point k of this thread (0 when k >= n^3).  Every thread of the CTA calls it.
-__device__ double eval_at_point(const double* F, double* T1, double* T2, const double* const* M, int d0, int d1,
-                                int d2, int n, int k) {
-    const int n2 = n * n, n3 = n2 * n;
-    const double* A = M[d0];
-    const double* B = M[d1];
-    const double* Z = M[d2];
-    for (int t = threadIdx.x; t < n3; t += blockDim.x) {
-        const int i = t % n, r = t / n;
-        double s = 0.0;
-        for (int m = 0; m < n; ++m) s += A[i * n + m] * F[m + n * r];
-        T1[t] = s;
+// The kernel is bound by FP64 arithmetic (two operations per clock and SM), so
+// it shares the partial passes of the derivatives (19 n^4 multiply-adds for the
+// value, gradient and Hessian of u instead of 30 n^4), contracts the block
+// map's second derivatives with the gradient before expanding them, divides
+// once per point and length, and leaves the mortar sums to one warp per slot.
+// 1,056 elements of the cubed sphere, n = 5..9: 1.75 -> 0.43 ms.
+
+struct Derivs {            // value, first and second reference derivatives (00, 11, 22, 01, 02, 12) at a point
+    double v, d[3], h[6];
+};
+
+// Derivatives of the nodal field F (n^3 values, x fastest) at GL point k of
+// this thread (0 when k >= n^3): value and gradient (LOW), Hessian (HIGH).
+// Every thread of the CTA calls it.
+template <bool LOW, bool HIGH>
+__device__ void eval_derivs(const double* F, double* T1, double* T2, const double* const* M, int n, int k, Derivs& o) {
+    const int n2 = n * n, n3 = n2 * n, ij = k % n2, l = k / n2;
+    auto zdot = [&](const double* T, const double* Z) {
+        double v = 0.0;
+        if (k < n3)
+            for (int m = 0; m < n; ++m) v += Z[l * n + m] * T[ij + n2 * m];
+        return v;
+    };
+    for (int d0 = 0; d0 < (HIGH ? 3 : 2); ++d0) {
+        const double* A = M[d0];
+        for (int t = threadIdx.x; t < n3; t += blockDim.x) {
+            const int i = t % n, r = t / n;
+            double s = 0.0;
+            for (int m = 0; m < n; ++m) s += A[i * n + m] * F[m + n * r];
+            T1[t] = s;
+        }
+        __syncthreads();
+        const int ny = (HIGH ? 3 : 2) - d0;   // derivatives along y: 0 .. ny - 1
+        for (int t = threadIdx.x; t < n3; t += blockDim.x) {
+            const int i = t % n, j = (t / n) % n, c = t / n2;
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+            for (int m = 0; m < n; ++m) {
+                const double v = T1[i + n * (m + n * c)];
+                s0 += M[0][j * n + m] * v;
+                if (ny > 1) s1 += M[1][j * n + m] * v;
+                if (ny > 2) s2 += M[2][j * n + m] * v;
+            }
+            T2[t] = s0;
+            if (ny > 1) T2[kNV + t] = s1;
+            if (ny > 2) T2[2 * kNV + t] = s2;
+        }
+        __syncthreads();
+        if (d0 == 0) {
+            if (LOW) {
+                o.v = zdot(T2, M[0]);
+                o.d[1] = zdot(T2 + kNV, M[0]);
+                o.d[2] = zdot(T2, M[1]);
+            }
+            if (HIGH) {
+                o.h[1] = zdot(T2 + 2 * kNV, M[0]);
+                o.h[2] = zdot(T2, M[2]);
+                o.h[5] = zdot(T2 + kNV, M[1]);
+            }
+        } else if (d0 == 1) {
+            if (LOW) o.d[0] = zdot(T2, M[0]);
+            if (HIGH) {
+                o.h[3] = zdot(T2 + kNV, M[0]);
+                o.h[4] = zdot(T2, M[1]);
+            }
+        } else {
+            o.h[0] = zdot(T2, M[0]);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < n3; t += blockDim.x) {
-        const int i = t % n, j = (t / n) % n, l = t / n2;
-        double s = 0.0;
-        for (int m = 0; m < n; ++m) s += B[j * n + m] * T1[i + n * (m + n * l)];
-        T2[t] = s;
+}
+
+// Block map at xi (the formulas of blocks.h with one division per length): J,
+// and what map_second needs for sum_i g_i d^2 x_i / dxi_l dxi_m.
+struct MapPoint {
+    double u[3], du[2][3], il, t, R, dR, ddR;
+    int t1, t2;
+};
+
+__device__ void map_first(const dg_block& B, const double xi[3], double J[3][3], MapPoint& p) {
+    if (B.kind == DG_BLOCK_HEX8) {
+        double x[3];
+        block_jacobian(B, xi, J, x);
+        return;
     }
-    __syncthreads();
-    double v = 0.0;
-    if (k < n3) {
-        const int ij = k % n2, l = k / n2;
-        for (int m = 0; m < n; ++m) v += Z[l * n + m] * T2[ij + n2 * m];
+    int d;
+    double sg, v[3];
+    wedge_frame(B.face, d, sg, p.t1, p.t2);
+    for (int i = 0; i < 3; ++i) v[i] = i == d ? sg : (i == p.t1 ? xi[0] : xi[1]);
+    p.il = 1.0 / sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+    for (int i = 0; i < 3; ++i) p.u[i] = v[i] * p.il;
+    const double ua = (p.t1 == 0 ? p.u[0] : (p.t1 == 1 ? p.u[1] : p.u[2])), ub = (p.t2 == 0 ? p.u[0] : (p.t2 == 1 ? p.u[1] : p.u[2]));
+    for (int i = 0; i < 3; ++i) {
+        p.du[0][i] = ((i == p.t1 ? 1.0 : 0.0) - p.u[i] * ua) * p.il;
+        p.du[1][i] = ((i == p.t2 ? 1.0 : 0.0) - p.u[i] * ub) * p.il;
     }
-    __syncthreads();
+    p.t = 0.5 * (xi[2] + 1.0);
+    if (B.kind == DG_BLOCK_WEDGE) {
+        const double s = (1.0 - p.t) * B.a, r = p.t * B.r;
+        for (int i = 0; i < 3; ++i) {
+            J[i][0] = (i == p.t1 ? s : 0.0) + r * p.du[0][i];
+            J[i][1] = (i == p.t2 ? s : 0.0) + r * p.du[1][i];
+            J[i][2] = 0.5 * (B.r * p.u[i] - B.a * v[i]);
+        }
+    } else {
+        const double i1 = 1.0 / B.r1, i2 = 1.0 / B.r2, k = i1 - i2;
+        p.R = 1.0 / ((1.0 - p.t) * i1 + p.t * i2);
+        p.dR = p.R * p.R * k;
+        p.ddR = 2.0 * p.R * p.dR * k;
+        for (int i = 0; i < 3; ++i) {
+            J[i][0] = p.R * p.du[0][i];
+            J[i][1] = p.R * p.du[1][i];
+            J[i][2] = 0.5 * p.dR * p.u[i];
+        }
+    }
+}
+
+// S[c] = sum_i g_i d^2 x_i / dxi_l dxi_m, pairs in the order of Derivs::h.
+__device__ void map_second(const dg_block& B, const double xi[3], const MapPoint& p, const double g[3], double S[6]) {
+    if (B.kind == DG_BLOCK_HEX8) {
+        double s01 = 0.0, s02 = 0.0, s12 = 0.0;
+        for (int c = 0; c < 8; ++c) {
+            const double q = g[0] * B.corners[c][0] + g[1] * B.corners[c][1] + g[2] * B.corners[c][2];
+            double f[3], df[3];
+            for (int k = 0; k < 3; ++k) {
+                const bool hi = (c >> k) & 1;
+                f[k] = hi ? 0.5 * (1.0 + xi[k]) : 0.5 * (1.0 - xi[k]);
+                df[k] = hi ? 0.5 : -0.5;
+            }
+            s01 += df[0] * df[1] * f[2] * q;
+            s02 += df[0] * f[1] * df[2] * q;
+            s12 += f[0] * df[1] * df[2] * q;
+        }
+        S[0] = S[1] = S[2] = 0.0;
+        S[3] = s01;
+        S[4] = s02;
+        S[5] = s12;
+        return;
+    }
+    auto at = [&](const double* w, int i) { return i == 0 ? w[0] : (i == 1 ? w[1] : w[2]); };
+    auto dot = [&](const double* w) { return g[0] * w[0] + g[1] * w[1] + g[2] * w[2]; };
+    const double gu = dot(p.u), g0 = dot(p.du[0]), g1 = dot(p.du[1]);
+    const double ua = at(p.u, p.t1), ub = at(p.u, p.t2);
+    const double s00 = -(2.0 * g0 * ua + gu * at(p.du[0], p.t1)) * p.il;   // g . d_a d_b u
+    const double s11 = -(2.0 * g1 * ub + gu * at(p.du[1], p.t2)) * p.il;
+    const double s01 = -(g1 * ua + gu * at(p.du[1], p.t1) + g0 * ub) * p.il;
+    if (B.kind == DG_BLOCK_WEDGE) {
+        const double r = p.t * B.r;
+        S[0] = r * s00;
+        S[1] = r * s11;
+        S[2] = 0.0;
+        S[3] = r * s01;
+        S[4] = 0.5 * (B.r * g0 - B.a * at(g, p.t1));
+        S[5] = 0.5 * (B.r * g1 - B.a * at(g, p.t2));
+    } else {
+        S[0] = p.R * s00;
+        S[1] = p.R * s11;
+        S[2] = 0.25 * p.ddR * gu;
+        S[3] = p.R * s01;
+        S[4] = 0.5 * p.dR * g0;
+        S[5] = 0.5 * p.dR * g1;
+    }
+}
+
+__device__ double det3(const double (&J)[3][3]) {
+    return J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) - J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
+           J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+}
+
+__device__ double warp_sum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Sum over the CTA, in a fixed order; the result is valid in thread 0.
+// Sum over the CTA, in a fixed order; the result is valid in warp 0.
 __device__ double block_sum(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();
+    v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    return s;
+    return threadIdx.x < 32 ? warp_sum(threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0) : 0.0;
 }
 
 __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, const double* u, const double* g,
@@ -79,9 +218,9 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
     if (e >= a.n_elems) return;
     const int n = a.p[e] + 1, n2 = n * n, n3 = n2 * n;
     const int k = threadIdx.x;
-    __shared__ double F[kNV], T1[kNV], T2[kNV];
+    __shared__ double F[kNV], T1[kNV], T2[3 * kNV];
     __shared__ double Mx[3][kMaxN * kMaxN];
-    __shared__ double red[32];
+    __shared__ double red[32], mort[kEstMaxSlots], V[8][3];
     const double* I = a.tab + tab_n(TabIndex::I, n);
     const double* D1 = a.tab + tab_n(TabIndex::IDg, n);
     const double* DL = a.tab + tab_n(TabIndex::DL, n);
@@ -99,78 +238,66 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
     const double* ue = u + a.dof_off[e];
     const bool blk = a.n_blocks > 0;
 
-    // element diameter: largest distance between two of the eight vertices
-    double he = 0.0;
+    // element diameter: largest distance between two of the eight vertices (a lane per vertex, then per pair)
+    double he2 = 0.0;
     double binv = 1.0, bxi0[3] = {0.0, 0.0, 0.0};   // block meshes: xi_block = bxi0 + binv (xi + 1)
     if (blk) {
         const int* lf = a.leaves + 4 * e;
         binv = 1.0 / (double)(1 << lf[0]);
         for (int dd = 0; dd < 3; ++dd) bxi0[dd] = -1.0 + 2.0 * lf[1 + dd] * binv;
     }
-    if (threadIdx.x == 0 && blk) {
-        const dg_block& BF = a.fblocks[a.block[e]];
-        double V[8][3];
-        for (int c = 0; c < 8; ++c) {
+    if (threadIdx.x < 32) {
+        const int c = threadIdx.x & 7;
+        double x[3];
+        if (blk) {
             double xb[3];
             for (int dd = 0; dd < 3; ++dd) xb[dd] = bxi0[dd] + binv * (((c >> dd) & 1) ? 2.0 : 0.0);
-            block_point(BF, xb, V[c]);
-        }
-        for (int c = 0; c < 8; ++c)
-            for (int d = c + 1; d < 8; ++d) {
-                const double dx = V[c][0] - V[d][0], dy = V[c][1] - V[d][1], dz = V[c][2] - V[d][2];
-                he = fmax(he, sqrt(dx * dx + dy * dy + dz * dz));
-            }
-    } else if (threadIdx.x == 0) {
-        double V[8][3];
-        for (int c = 0; c < 8; ++c) {
+            block_point(a.fblocks[a.block[e]], xb, x);
+        } else {
             const int idx = ((c & 1) ? n - 1 : 0) + n * (((c >> 1) & 1) ? n - 1 : 0) + n2 * (((c >> 2) & 1) ? n - 1 : 0);
-            for (int i = 0; i < 3; ++i) V[c][i] = Xe[i * n3 + idx];
+            for (int i = 0; i < 3; ++i) x[i] = Xe[i * n3 + idx];
         }
-        for (int c = 0; c < 8; ++c)
-            for (int d = c + 1; d < 8; ++d) {
-                const double dx = V[c][0] - V[d][0], dy = V[c][1] - V[d][1], dz = V[c][2] - V[d][2];
-                he = fmax(he, sqrt(dx * dx + dy * dy + dz * dz));
-            }
+        if (threadIdx.x < 8)
+            for (int i = 0; i < 3; ++i) V[c][i] = x[i];
+        __syncwarp();
+        for (int p = threadIdx.x; p < 64; p += 32) {
+            const double dx = V[p & 7][0] - V[p >> 3][0], dy = V[p & 7][1] - V[p >> 3][1], dz = V[p & 7][2] - V[p >> 3][2];
+            he2 = fmax(he2, dx * dx + dy * dy + dz * dz);
+        }
+        for (int o = 16; o > 0; o >>= 1) he2 = fmax(he2, __shfl_xor_sync(0xffffffffu, he2, o));
     }
+    __syncthreads();
 
-    // J_il = d x_i / d xi_l (and, on block meshes, the map's second derivatives Xs and the
-    // fiducial Jacobian determinant of the volume weight)
-    double J[3][3], Xs[3][3][3], detW = 0.0;
+    // J_il = d x_i / d xi_l (block meshes: the exact map's) and the fiducial Jacobian
+    // determinant of the volume weight
+    double J[3][3], xb[3] = {0.0, 0.0, 0.0}, detW = 0.0;
+    MapPoint mp;
+    Derivs D;
     if (blk) {
-        double xp[3], xb[3] = {0.0, 0.0, 0.0};
         const double* xg = a.tab + tab_n(TabIndex::GLx, n);
         if (k < n3) {
             const int ii[3] = {k % n, (k / n) % n, k / n2};
             for (int dd = 0; dd < 3; ++dd) xb[dd] = bxi0[dd] + binv * (xg[ii[dd]] + 1.0);
-        }
-        const dg_block& B = a.blocks[a.block[e]];
-        block_jacobian(B, xb, J, xp);
-        block_hessian(B, xb, Xs);
-        for (int i = 0; i < 3; ++i)
-            for (int l = 0; l < 3; ++l) {
-                J[i][l] *= binv;
-                for (int m = 0; m < 3; ++m) Xs[i][l][m] *= binv * binv;
+            if (a.fblocks != a.blocks) {
+                map_first(a.fblocks[a.block[e]], xb, J, mp);
+                detW = det3(J) * (binv * binv * binv);
             }
-        double JF[3][3];
-        block_jacobian(a.fblocks[a.block[e]], xb, JF, xp);
-        for (int i = 0; i < 3; ++i)
-            for (int l = 0; l < 3; ++l) JF[i][l] *= binv;
-        detW = JF[0][0] * (JF[1][1] * JF[2][2] - JF[1][2] * JF[2][1]) -
-               JF[0][1] * (JF[1][0] * JF[2][2] - JF[1][2] * JF[2][0]) +
-               JF[0][2] * (JF[1][0] * JF[2][1] - JF[1][1] * JF[2][0]);
+            map_first(a.blocks[a.block[e]], xb, J, mp);
+            for (int i = 0; i < 3; ++i)
+                for (int l = 0; l < 3; ++l) J[i][l] *= binv;
+        }
     } else {
         for (int i = 0; i < 3; ++i) {
             for (int t = threadIdx.x; t < n3; t += blockDim.x) F[t] = Xe[i * n3 + t];
             __syncthreads();
-            J[i][0] = eval_at_point(F, T1, T2, M, 1, 0, 0, n, k);
-            J[i][1] = eval_at_point(F, T1, T2, M, 0, 1, 0, n, k);
-            J[i][2] = eval_at_point(F, T1, T2, M, 0, 0, 1, n, k);
+            eval_derivs<true, false>(F, T1, T2, M, n, k, D);
+            for (int l = 0; l < 3; ++l) J[i][l] = D.d[l];
         }
     }
     double Ji[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}}, det = 1.0;
     if (k < n3) {
-        det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) - J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-              J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+        det = det3(J);
+        if (!blk || a.fblocks == a.blocks) detW = det;
         const double r = 1.0 / det;
         Ji[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) * r;
         Ji[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * r;
@@ -183,31 +310,27 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
         Ji[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * r;
     }
 
-    // u, its physical gradient and the reference Hessian; pairs (l, m) in the
-    // order 00, 11, 22, 01, 02, 12
-    constexpr int kD[6][3] = {{2, 0, 0}, {0, 2, 0}, {0, 0, 2}, {1, 1, 0}, {1, 0, 1}, {0, 1, 1}};
+    // u, its physical gradient and the reference Hessian
     for (int t = threadIdx.x; t < n3; t += blockDim.x) F[t] = ue[t];
     __syncthreads();
-    const double uv = eval_at_point(F, T1, T2, M, 0, 0, 0, n, k);
-    double du[3];
-    du[0] = eval_at_point(F, T1, T2, M, 1, 0, 0, n, k);
-    du[1] = eval_at_point(F, T1, T2, M, 0, 1, 0, n, k);
-    du[2] = eval_at_point(F, T1, T2, M, 0, 0, 1, n, k);
-    double ux[3];
-    for (int i = 0; i < 3; ++i) ux[i] = Ji[0][i] * du[0] + Ji[1][i] * du[1] + Ji[2][i] * du[2];
-    double H[6];
-    for (int c = 0; c < 6; ++c) H[c] = eval_at_point(F, T1, T2, M, kD[c][0], kD[c][1], kD[c][2], n, k);
+    eval_derivs<true, true>(F, T1, T2, M, n, k, D);
+    const double uv = D.v;
+    double ux[3], H[6];
+    for (int i = 0; i < 3; ++i) ux[i] = Ji[0][i] * D.d[0] + Ji[1][i] * D.d[1] + Ji[2][i] * D.d[2];
+    for (int c = 0; c < 6; ++c) H[c] = D.h[c];
     // minus sum_k (du/dx_k) X^k
     if (blk) {
-        constexpr int kLM[6][2] = {{0, 0}, {1, 1}, {2, 2}, {0, 1}, {0, 2}, {1, 2}};
-        for (int i = 0; i < 3; ++i)
-            for (int c = 0; c < 6; ++c) H[c] -= ux[i] * Xs[i][kLM[c][0]][kLM[c][1]];
+        if (k < n3) {
+            double S[6];
+            map_second(a.blocks[a.block[e]], xb, mp, ux, S);
+            for (int c = 0; c < 6; ++c) H[c] -= S[c] * (binv * binv);
+        }
     } else {
         for (int i = 0; i < 3; ++i) {
             for (int t = threadIdx.x; t < n3; t += blockDim.x) F[t] = Xe[i * n3 + t];
             __syncthreads();
-            for (int c = 0; c < 6; ++c)
-                H[c] -= ux[i] * eval_at_point(F, T1, T2, M, kD[c][0], kD[c][1], kD[c][2], n, k);
+            eval_derivs<false, true>(F, T1, T2, M, n, k, D);
+            for (int c = 0; c < 6; ++c) H[c] -= ux[i] * D.h[c];
         }
     }
     double vol = 0.0;
@@ -220,20 +343,20 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
         const long long vo = a.vqp_off[e];
         const double R = (f ? f[vo + k] : 0.0) * uv - (g ? g[vo + k] : 0.0) - lap;
         const double w = wg[k % n] * wg[(k / n) % n] * wg[k / n2];
-        vol = w * (blk ? detW : det) * R * R;
+        vol = w * detW * R * R;
     }
     vol = block_sum(vol, red);
 
-    // mortar terms of the element's slots
-    double mort = 0.0;
-    for (int s = a.slot_off[e]; s < a.slot_off[e + 1]; ++s) {
-        const int mi = a.slot_mortar[s];
+    // mortar terms of the element's slots, a warp per slot, summed in slot order
+    const int s0 = a.slot_off[e], ns = a.slot_off[e + 1] - s0, lane = threadIdx.x & 31;
+    for (int s = threadIdx.x >> 5; s < ns && s < kEstMaxSlots; s += blockDim.x >> 5) {
+        const int mi = a.slot_mortar[s0 + s];
         const Mortar Mo = a.mortars[mi];
         const int q2 = Mo.q * Mo.q;
         const double* mg = a.mgW + 7 * Mo.goff;   // w S of the weighting grid
         const double* mt = a.mt + 4 * Mo.goff;
         double s1 = 0.0, s2 = 0.0;
-        for (int pt = threadIdx.x; pt < q2; pt += blockDim.x) {
+        for (int pt = lane; pt < q2; pt += 32) {
             const double wS = mg[pt];
             if (Mo.eB >= 0) {
                 const double j1 = mt[q2 + pt] - mt[3 * q2 + pt];
@@ -245,17 +368,20 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
                 s2 += wS * j3 * j3;
             }
         }
-        s1 = block_sum(s1, red);
-        s2 = block_sum(s2, red);
-        if (threadIdx.x == 0) {
+        s1 = warp_sum(s1);
+        s2 = warp_sum(s2);
+        if (lane == 0) {
             const double pm = Mo.q - 1, sig = a.sigW[mi];
             const double hm = a.C * pm * pm / sig;
-            mort += (Mo.eB >= 0 ? hm / pm * s1 : 0.0) + sig / hm * pm * pm * s2;
+            mort[s] = (Mo.eB >= 0 ? hm / pm * s1 : 0.0) + sig / hm * pm * pm * s2;
         }
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
         const double pe = n - 1;
-        eta2[e] = he * he * pe * pe * vol + mort;
+        double m = 0.0;
+        for (int s = 0; s < ns && s < kEstMaxSlots; ++s) m += mort[s];
+        eta2[e] = he2 * pe * pe * vol + m;
     }
 }
 
