@@ -18,6 +18,7 @@ __global__ void rhs_kernel(RhsArgs a, const double* g, const double* gD, double*
     if (e >= a.n_elems) return;
     const int n = a.p[e] + 1, n2 = n * n, n3 = n2 * n;
     __shared__ double b0[kMaxN * kMaxN * kMaxN], b1[kMaxN * kMaxN * kMaxN], Fe[kMaxN * kMaxN * kMaxN];
+    __shared__ double P[4 * kMaxN * kMaxN], X[3 * kMaxN * kMaxN];
     const double* I = a.tab + tab_n(TabIndex::I, n);
     const long long vo = a.vqp_off[e];
     for (int k = threadIdx.x; k < n3; k += blockDim.x) b0[k] = g ? a.wdetJ[vo + k] * g[vo + k] : 0.0;
@@ -58,17 +59,40 @@ __global__ void rhs_kernel(RhsArgs a, const double* g, const double* gD, double*
             const double* Dm = a.tab + tab_m(TabIndex::Dm, n, q, 0);
             const double* mg = a.mg + 7 * M.goff;
             const double sig = a.sigma[a.slot_mortar[s]];
+            // flux factors at the mortar points, then lifted direction by direction (FP64 arithmetic bounds
+            // the kernel: 7 q n^2 multiply-adds a face instead of 10 q^2 n^2 point by point)
+            double *PA = P, *P1 = PA + q2, *P2 = P1 + q2, *Pn = P2 + q2;
+            for (int pt = threadIdx.x; pt < q2; pt += blockDim.x) {
+                const double v = mg[pt] * gD[M.bnd_off + pt];
+                PA[pt] = sig * v;
+                P1[pt] = -v * mg[(1 + t1) * q2 + pt];
+                P2[pt] = -v * mg[(1 + t2) * q2 + pt];
+                Pn[pt] = -v * mg[(1 + d) * q2 + pt];
+            }
+            __syncthreads();
+            double *X1 = X, *X2 = X1 + q * n, *X3 = X2 + q * n;
+            for (int k = threadIdx.x; k < q * n; k += blockDim.x) {
+                const int i1 = k % q, bb = k / q;
+                double x1 = 0.0, x2 = 0.0, x3 = 0.0;
+                for (int i2 = 0; i2 < q; ++i2) {
+                    const double iv = Im[i2 * n + bb], dv = Dm[i2 * n + bb];
+                    const int pt = i1 + q * i2;
+                    x1 += iv * PA[pt] + dv * P2[pt];
+                    x2 += iv * P1[pt];
+                    x3 += iv * Pn[pt];
+                }
+                X1[k] = x1;
+                X2[k] = x2;
+                X3[k] = x3;
+            }
+            __syncthreads();
             for (int k = threadIdx.x; k < n2; k += blockDim.x) {
                 const int aa = k % n, bb = k / n;
                 double fu = 0.0, fd = 0.0;
-                for (int pt = 0; pt < q2; ++pt) {
-                    const int i1 = pt % q, i2 = pt / q;
-                    const double wS = mg[pt], gd = gD[M.bnd_off + pt];
-                    const double A = wS * sig * gd, B = -wS * gd;
-                    const double c1 = mg[(1 + t1) * q2 + pt], c2 = mg[(1 + t2) * q2 + pt], cd = mg[(1 + d) * q2 + pt];
-                    const double I1 = Im[i1 * n + aa], I2 = Im[i2 * n + bb];
-                    fu += A * I1 * I2 + B * (c1 * Dm[i1 * n + aa] * I2 + c2 * I1 * Dm[i2 * n + bb]);
-                    fd += B * cd * I1 * I2;
+                for (int i1 = 0; i1 < q; ++i1) {
+                    const double iv = Im[i1 * n + aa], dv = Dm[i1 * n + aa];
+                    fu += iv * X1[i1 + q * bb] + dv * X2[i1 + q * bb];
+                    fd += iv * X3[i1 + q * bb];
                 }
                 const int base = aa * st[t1] + bb * st[t2];
                 Fe[base + fn * st[d]] += fu;
