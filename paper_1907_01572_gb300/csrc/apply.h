@@ -33,6 +33,18 @@ template <typename T>
 cudaError_t launch_apply(const LevelView<T>& L, const BucketInfo* buckets, const T* x, T* y, cudaStream_t st,
                          int* launches, int* plan = nullptr, const ApplyStreams* as = nullptr);
 
+// FP64 with the contractions on the tensor pipe (apply_f64x.cuh): levels of at
+// least kX64MinElems elements, two per SM.  Smaller (coarse) levels keep the
+// native kernels and so their results bit for bit: the V-cycle with the CG
+// eigenvalue estimate can amplify rounding 1e8 times on them (the stretched
+// cubed sphere at level 1), and a preconditioner should not move with it.
+// Up to kX64FusedMaxElems elements the degrees share one launch (960 hp elements:
+// 126 us against 251 in a launch per degree; 7,680: 642 against 571).
+constexpr int kX64MinElems = 305;
+constexpr int kX64FusedMaxElems = 2048;
+cudaError_t launch_apply_x64(const LevelView<double>& L, const BucketInfo* buckets, const double* x, double* y,
+                             cudaStream_t st, int* launches, const ApplyStreams* as);
+
 // BF16 operand x (2-byte bfloat16 values), FP32 arithmetic and FP32 y.
 cudaError_t launch_apply_bf16(const LevelView<float>& L, const BucketInfo* buckets, const void* x, float* y,
                               cudaStream_t st, int* launches, int* plan = nullptr,

@@ -1320,14 +1320,11 @@ cudaError_t launch_fused_cta(const LevelView<T>& L, const BucketInfo* buckets, c
 
 }  // namespace apply_detail
 
-template <typename T, typename TX>
-cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
-                        cudaStream_t st, int* launches, const ApplyStreams* as) {
-    if (path == 0) return apply_detail::launch_fused_cta<T, TX>(L, buckets, x, y, st, launches);
-    if (path == 1) return apply_detail::launch_fused_warp<T, TX>(L, buckets, x, y, st, launches);
-    // Per-bucket launches, largest bucket (elements x n^3) first; plan 3 deals
-    // them round robin over the caller's stream and the side streams.
-    if (path == 2) as = nullptr;
+// Per-bucket launches, largest bucket (elements x n^3) first, dealt round robin
+// over the caller's stream and the side streams (as, or none): fn(phase, n,
+// stream) for the trace phase (0), then the element phase (1).
+template <typename FN>
+cudaError_t for_buckets(const BucketInfo* buckets, cudaStream_t st, int* launches, const ApplyStreams* as, FN fn) {
     int order[kNumN], nb = 0;
     for (int n = kMinN; n <= kMaxN; ++n)
         if (buckets[n].count > 0) order[nb++] = n;
@@ -1341,21 +1338,8 @@ cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* bu
             if (err != cudaSuccess) return err;
         }
         for (int j = 0; j < nb; ++j) {
-            const int n = order[j], k = j % (ns + 1);
-            const cudaStream_t sj = k == 0 ? st : as->side[k - 1];
-            const BucketInfo& b = buckets[n];
-            cudaError_t err = cudaSuccess;
-            if (phase == 0 && L.oriented) {
-                DG_N_SWITCH(n, (err = apply_detail::launch_trace<NN, T, TX, true>(L, b, x, sj)))
-            } else if (phase == 0) {
-                DG_N_SWITCH(n, (err = apply_detail::launch_trace<NN, T, TX, false>(L, b, x, sj)))
-            } else if (L.bdiag) {   // block-diagonal apply: the general (turned-interface) form
-                DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, true, true>(L, b, x, y, sj)))
-            } else if (L.oriented) {
-                DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, true>(L, b, x, y, sj)))
-            } else {
-                DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, false>(L, b, x, y, sj)))
-            }
+            const int k = j % (ns + 1);
+            const cudaError_t err = fn(phase, order[j], k == 0 ? st : as->side[k - 1]);
             if (err != cudaSuccess) return err;
             if (launches) ++*launches;
         }
@@ -1366,6 +1350,29 @@ cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* bu
         }
     }
     return cudaSuccess;
+}
+
+template <typename T, typename TX>
+cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y,
+                        cudaStream_t st, int* launches, const ApplyStreams* as) {
+    if (path == 0) return apply_detail::launch_fused_cta<T, TX>(L, buckets, x, y, st, launches);
+    if (path == 1) return apply_detail::launch_fused_warp<T, TX>(L, buckets, x, y, st, launches);
+    return for_buckets(buckets, st, launches, path == 2 ? nullptr : as, [&](int phase, int n, cudaStream_t sj) {
+        const BucketInfo& b = buckets[n];
+        cudaError_t err = cudaSuccess;
+        if (phase == 0 && L.oriented) {
+            DG_N_SWITCH(n, (err = apply_detail::launch_trace<NN, T, TX, true>(L, b, x, sj)))
+        } else if (phase == 0) {
+            DG_N_SWITCH(n, (err = apply_detail::launch_trace<NN, T, TX, false>(L, b, x, sj)))
+        } else if (L.bdiag) {   // block-diagonal apply: the general (turned-interface) form
+            DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, true, true>(L, b, x, y, sj)))
+        } else if (L.oriented) {
+            DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, true>(L, b, x, y, sj)))
+        } else {
+            DG_N_SWITCH(n, (err = apply_detail::launch_element<NN, T, TX, false>(L, b, x, y, sj)))
+        }
+        return err;
+    });
 }
 
 template <typename T, typename TX>
@@ -1395,6 +1402,9 @@ inline int forced_plan() {
 template <typename T, typename TX>
 cudaError_t launch_apply_x(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y, cudaStream_t st,
                            int* launches, int* plan, const ApplyStreams* as = nullptr) {
+    if constexpr (sizeof(T) == 8)
+        if (L.x64.w != nullptr && L.n_elems >= kX64MinElems && !L.bdiag && forced_plan() < 0)
+            return launch_apply_x64(L, buckets, x, y, st, launches, as);
     int path = L.n_elems <= apply_detail::kCtaMaxElems ? 0 : (L.n_elems <= apply_detail::kFusedMaxElems ? 1 : 2);
     if (plan && *plan >= 0) return launch_path<T, TX>(*plan, L, buckets, x, y, st, launches, as);
     if (plan && forced_plan() >= 0) {

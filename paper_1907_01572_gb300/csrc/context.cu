@@ -13,6 +13,7 @@
 #include "geom.h"
 #include "source.h"
 #include "estimate.h"
+#include "f64x_tables.h"
 
 using namespace dg;
 
@@ -74,6 +75,7 @@ LevelView<double> level_view<double>(dg_ctx* c, int l) {
     v.ob_total = (long long)L.ob_count;
     v.oriented = L.oriented;
     v.chk = device_check_flag();
+    v.x64 = X64Tabs{c->x64_w, c->x64_s};
     v.mt = L.mt64;
     return v;
 }
@@ -1105,6 +1107,26 @@ int check_bc(const dg_mesh_desc* d, const BlockTopo& topo, std::string& err) {
     return DG_OK;
 }
 
+// The 1-D, mortar and digit tables (the same for every context), built once.
+struct HostTabs {
+    std::vector<double> tab, ftab;
+    std::vector<float> tabf, ftabf;
+    std::vector<unsigned> x64_w;
+    std::vector<int> x64_s;
+    bool x64_ok = false;
+    HostTabs() {
+        build_tables(tab);
+        build_face_tables(tab, ftab);
+        tabf.assign(tab.begin(), tab.end());
+        ftabf.assign(ftab.begin(), ftab.end());
+        x64_ok = build_x64_tables(tab, x64_w, x64_s);
+    }
+};
+const HostTabs& host_tabs() {
+    static const HostTabs t;   // thread-safe initialisation
+    return t;
+}
+
 size_t level_bytes(const LevelHost& h) {
     const size_t nv = h.vqp_off.back(), nd = h.n_dofs(), nm = h.n_mortar_pts;
     size_t b = 0;
@@ -1180,16 +1202,15 @@ int dg_ctx_create(const dg_mesh* mesh, const dg_disc_opts* opts, void* stream, d
     c->desc = mesh->desc;
     c->blocks = mesh->blocks;
     c->topo = mesh->topo;
-    std::vector<double> tab;
-    build_tables(tab);
-    std::vector<float> tabf(tab.begin(), tab.end());
-    c->tab64 = c->arena.upload(tab, c->st);
-    c->tab32 = c->arena.upload(tabf, c->st);
-    std::vector<double> ftab;
-    build_face_tables(tab, ftab);
-    std::vector<float> ftabf(ftab.begin(), ftab.end());
-    c->ftab64 = c->arena.upload(ftab, c->st);
-    c->ftab32 = c->arena.upload(ftabf, c->st);
+    const HostTabs& ht = host_tabs();
+    c->tab64 = c->arena.upload(ht.tab, c->st);
+    c->tab32 = c->arena.upload(ht.tabf, c->st);
+    if (ht.x64_ok) {
+        c->x64_w = c->arena.upload(ht.x64_w, c->st);
+        c->x64_s = c->arena.upload(ht.x64_s, c->st);
+    }
+    c->ftab64 = c->arena.upload(ht.ftab, c->st);
+    c->ftab32 = c->arena.upload(ht.ftabf, c->st);
     if (!c->blocks.empty()) c->blocks_dev = c->arena.upload(c->blocks, c->st);
     c->red.partials = c->arena.alloc<double>(kRedBlocks * 4);
     c->red.out = c->arena.alloc<double>(4);

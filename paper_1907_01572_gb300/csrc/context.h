@@ -110,6 +110,8 @@ struct dg_ctx {
     float* tab32 = nullptr;
     double* ftab64 = nullptr;
     float* ftab32 = nullptr;
+    unsigned* x64_w = nullptr;      // digit tables of the FP64 apply on the tensor pipe (f64x_tables.h)
+    int* x64_s = nullptr;
     dg::Red red{};
     double* red_host = nullptr;     // pinned, 4 doubles
     dg::FcgState* fcg = nullptr;

@@ -137,6 +137,11 @@ struct SlotPack {
     long long goff;
 };
 
+struct X64Tabs {           // digit tables of f64x_tables.h (device); w == nullptr: not available
+    const unsigned* w;
+    const int* s;
+};
+
 template <typename T>
 struct LevelView {         // passed by value to kernels
     int n_elems;
@@ -161,6 +166,7 @@ struct LevelView {         // passed by value to kernels
     int oriented;          // some mortar of the level has a turned side B (Mortar::orient != 0)
     int bdiag;             // apply only the element diagonal blocks (the neighbour's trace taken as 0)
     int* chk;              // self-check flag
+    X64Tabs x64;           // FP64 views only
     T* mt;                 // mortar trace buffer: 4 * n_mortar_pts ([u_A, dn_A, u_B, dn_B] per mortar)
 };
 
