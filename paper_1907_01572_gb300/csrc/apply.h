@@ -33,6 +33,14 @@ template <typename T>
 cudaError_t launch_apply(const LevelView<T>& L, const BucketInfo* buckets, const T* x, T* y, cudaStream_t st,
                          int* launches, int* plan = nullptr, const ApplyStreams* as = nullptr);
 
+// Levels of at most this many elements (four per SM) hold the neighbours' records
+// that the one-launch FP32 apply (apply_one.cuh) needs; whether it is the fastest
+// on a level is measured with the other plans.  Alone it is faster beyond (1,056
+// elements: 58 us against 65), but there the traces computed twice cost other
+// streams their share: with three contexts in flight 832 elements took 41 us a
+// pass against 33, 512 elements 15.0 against 15.7.
+constexpr int kOneMaxElems = 608;
+
 // FP64 with the contractions on the tensor pipe (apply_f64x.cuh): levels of at
 // least kX64MinElems elements, two per SM.  Smaller (coarse) levels keep the
 // native kernels and so their results bit for bit: the V-cycle with the CG

@@ -1320,6 +1320,12 @@ cudaError_t launch_fused_cta(const LevelView<T>& L, const BucketInfo* buckets, c
 
 }  // namespace apply_detail
 
+}  // namespace dg
+
+#include "apply_one.cuh"
+
+namespace dg {
+
 // Per-bucket launches, largest bucket (elements x n^3) first, dealt round robin
 // over the caller's stream and the side streams (as, or none): fn(phase, n,
 // stream) for the trace phase (0), then the element phase (1).
@@ -1357,6 +1363,8 @@ cudaError_t launch_kernels(int path, const LevelView<T>& L, const BucketInfo* bu
                         cudaStream_t st, int* launches, const ApplyStreams* as) {
     if (path == 0) return apply_detail::launch_fused_cta<T, TX>(L, buckets, x, y, st, launches);
     if (path == 1) return apply_detail::launch_fused_warp<T, TX>(L, buckets, x, y, st, launches);
+    if constexpr (sizeof(T) == 4)
+        if (path == 4) return apply_detail::launch_one<T, TX>(L, buckets, x, y, st, launches);
     return for_buckets(buckets, st, launches, path == 2 ? nullptr : as, [&](int phase, int n, cudaStream_t sj) {
         const BucketInfo& b = buckets[n];
         cudaError_t err = cudaSuccess;
@@ -1387,7 +1395,8 @@ cudaError_t launch_path(int path, const LevelView<T>& L, const BucketInfo* bucke
 
 // Launch plan of a level: 0 one CTA per element, 1 one warp per element in a
 // single launch per kernel, 2 per-degree-bucket launches with occupancy-sized
-// CTAs, 3 the same spread over side streams.  With a plan slot and outside
+// CTAs, 3 the same spread over side streams, 4 (FP32, small levels) everything
+// in one launch (apply_one.cuh).  With a plan slot and outside
 // stream capture the first apply times the candidates (each writes the same
 // outputs, in the same order of summation) and keeps the fastest; otherwise a
 // size rule picks.  DGELL_APPLY_PLAN=0..3 fixes the plan of every tuned level.
@@ -1406,6 +1415,8 @@ cudaError_t launch_apply_x(const LevelView<T>& L, const BucketInfo* buckets, con
         if (L.x64.w != nullptr && L.n_elems >= kX64MinElems && !L.bdiag && forced_plan() < 0)
             return launch_apply_x64(L, buckets, x, y, st, launches, as);
     int path = L.n_elems <= apply_detail::kCtaMaxElems ? 0 : (L.n_elems <= apply_detail::kFusedMaxElems ? 1 : 2);
+    const bool one = sizeof(T) == 4 && L.snb != nullptr;
+    if (one && L.n_elems <= 2 * apply_detail::kCtaMaxElems) path = 4;
     if (plan && *plan >= 0) return launch_path<T, TX>(*plan, L, buckets, x, y, st, launches, as);
     if (plan && forced_plan() >= 0) {
         *plan = forced_plan();
@@ -1431,8 +1442,8 @@ cudaError_t launch_apply_x(const LevelView<T>& L, const BucketInfo* buckets, con
         cudaEventCreate(&e1);
         float best = 1e30f;
         int best_path = path;
-        const int ncand = (as && as->n > 0) ? 4 : 3;
-        for (int cand = 0; cand < ncand; ++cand) {
+        for (int cand = 0; cand <= 4; ++cand) {
+            if ((cand == 3 && !(as && as->n > 0)) || (cand == 4 && !one)) continue;
             cudaError_t err = launch_path<T, TX>(cand, L, buckets, x, y, st, nullptr, as);   // warm-up / validity
             if (err != cudaSuccess) {
                 cudaGetLastError();

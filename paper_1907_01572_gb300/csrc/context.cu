@@ -98,6 +98,7 @@ LevelView<float> level_view<float>(dg_ctx* c, int l) {
     v.slot_side = L.slot_side;
     v.mortars = L.mortars;
     v.spack = L.spack32;
+    v.snb = L.snb;
     v.mg = L.mg32;
     v.sigma = L.sigma32;
     v.tab = c->tab32;
@@ -1005,6 +1006,20 @@ int upload_level(dg_ctx* c, LevelDev& L, int li, std::string& err) {
         }
         std::vector<SlotPack<float>> sp32(sp.size());
         for (size_t s = 0; s < sp.size(); ++s) sp32[s] = SlotPack<float>{sp[s].info, 0.f, sp[s].goff};
+        if (h.n_elems() <= kOneMaxElems) {
+            std::vector<SlotNb> nb(sp.size());
+            for (size_t s = 0; s < sp.size(); ++s) {
+                const Mortar& m = h.mortars[h.slot_mortar[s]];
+                const bool isA = h.slot_side[s] == 0;   // the other side is B
+                const int e2 = isA ? m.eB : m.eA;
+                if (e2 < 0) continue;
+                const int f = isA ? m.fB : m.fA, p0 = isA ? m.posB0 : m.posA0, p1 = isA ? m.posB1 : m.posA1;
+                nb[s].dofo = h.dof_off[e2];
+                nb[s].info = f | p0 << 4 | p1 << 6 | (isA ? (int)m.orient << 13 : 0);
+                nb[s].n = h.p[e2] + 1;
+            }
+            L.snb = A.upload(nb, st);
+        }
         L.spack64 = A.upload(sp, st);
         L.spack32 = A.upload(sp32, st);
     }

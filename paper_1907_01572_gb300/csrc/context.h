@@ -65,6 +65,7 @@ struct LevelDev {
     Mortar* mortars = nullptr;
     int *slot_off = nullptr, *slot_mortar = nullptr;
     unsigned char *slot_face = nullptr, *slot_side = nullptr;
+    SlotNb* snb = nullptr;            // other side of every slot (levels of at most kOneMaxElems elements)
     SlotPack<double>* spack64 = nullptr;
     SlotPack<float>* spack32 = nullptr;
     BucketInfo buckets[kMaxN + 1] = {};

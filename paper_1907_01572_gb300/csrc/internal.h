@@ -137,6 +137,14 @@ struct SlotPack {
     long long goff;
 };
 
+// The other side of a mortar slot, for kernels that read the neighbour's values
+// themselves: its DOF offset, its face, sub-face positions and orientation
+// (bits as in SlotPack::info) and its n = p + 1 (0 on the boundary).
+struct SlotNb {
+    long long dofo;
+    int info, n;
+};
+
 struct X64Tabs {           // digit tables of f64x_tables.h (device); w == nullptr: not available
     const unsigned* w;
     const int* s;
@@ -158,6 +166,7 @@ struct LevelView {         // passed by value to kernels
     const unsigned char* slot_side;
     const Mortar* mortars;
     const SlotPack<T>* spack;   // per slot, in slot order
+    const SlotNb* snb;     // per slot (small levels, see kOneMaxElems; else nullptr)
     const T* mg;           // 7 * n_mortar_pts: [wS, cA0, cA1, cA2, cB0, cB1, cB2] blocks per mortar
     const T* sigma;        // per mortar
     const T* tab;
