@@ -190,17 +190,43 @@ __device__ __forceinline__ void pass_rows(const T* __restrict__ in, T* __restric
     }
 }
 
-// out = M in along direction DIR of an N^3 array held by nt threads (TRANS: M^T; ACC: out +=);
-// M points at the padded rows of the operator, its transpose follows.
+// The pass on more threads than pencils (nt > N^2): the outputs of a pencil are
+// shared by nt / N^2 threads.  With a thread per pencil the 64 pencils of n = 8
+// sat on two of an SM's four quarters, and in FP64, where a quarter issues half a
+// value per clock, the pass took twice the time of the whole SM (FP64 apply of 64
+// elements, p = 5: 38.9 -> 30.0 us).  Every output is the same sum in the same
+// order as in pass_rows.
+template <int N, int DIR, bool ACC, typename T>
+__device__ __forceinline__ void pass_split(const T* __restrict__ in, T* __restrict__ out, const T* __restrict__ R,
+                                           int t, int nt) {
+    constexpr int NP = r4(N), S1 = Strides<N>::S1, S2 = Strides<N>::S2;
+    constexpr int stride = DIR == 0 ? 1 : (DIR == 1 ? S1 : S2);
+    const int share = nt / (N * N), per = (N + share - 1) / share, pid = t % (N * N), i0 = t / (N * N) * per;
+    if (i0 >= N) return;
+    const int u = pid % N, w = pid / N;
+    const int base = DIR == 0 ? S1 * u + S2 * w : (DIR == 1 ? u + S2 * w : u + S1 * w);
+    T v[N];
+#pragma unroll
+    for (int m = 0; m < N; ++m) v[m] = in[base + m * stride];
+    for (int i = i0; i < min(N, i0 + per); ++i) {
+        T r[N], s = 0;
+        load_row<N>(R + i * NP, r);
+#pragma unroll
+        for (int m = 0; m < N; ++m) s += r[m] * v[m];
+        if (ACC) out[base + i * stride] += s;
+        else out[base + i * stride] = s;
+    }
+}
+
+// out = M in along direction DIR of an N^3 array held by nt threads, 32 or more
+// than N^2 (TRANS: M^T; ACC: out +=); M points at the padded rows of the
+// operator, its transpose follows.
 template <int N, int DIR, bool TRANS, bool ACC, typename T>
 __device__ inline void wpass(const T* __restrict__ in, T* __restrict__ out, const T* __restrict__ M, int t,
                              int nt = 32) {
     const T* R = TRANS ? M + N * r4(N) : M;
-    if (nt == 32) {
-        pass_rows<N, DIR, ACC, (N * N + 31) / 32>(in, out, R, t, 32);
-    } else {
-        for (int t0 = t; t0 < N * N; t0 += nt) pass_rows<N, DIR, ACC, 1>(in, out, R, t0, nt);
-    }
+    if (nt == 32) pass_rows<N, DIR, ACC, (N * N + 31) / 32>(in, out, R, t, 32);
+    else pass_split<N, DIR, ACC>(in, out, R, t, nt);
 }
 
 // ---- tensor-core passes (FP32 and BF16-operand applies, N <= 8) -------------
