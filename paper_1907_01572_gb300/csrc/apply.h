@@ -42,14 +42,37 @@ cudaError_t launch_apply(const LevelView<T>& L, const BucketInfo* buckets, const
 constexpr int kOneMaxElems = 608;
 
 // FP64 with the contractions on the tensor pipe (apply_f64x.cuh): levels of at
-// least kX64MinElems elements, two per SM.  Smaller (coarse) levels keep the
-// native kernels and so their results bit for bit: the V-cycle with the CG
-// eigenvalue estimate can amplify rounding 1e8 times on them (the stretched
-// cubed sphere at level 1), and a preconditioner should not move with it.
+// least kX64MinElems elements, two per SM, where the chip is full enough for the
+// digits' throughput to count more than an element's latency (512 elements of p =
+// 3: 41 us against 64 of the native kernels; 216 are no longer two per SM).  On
+// those below, the native kernels also keep their results bit for bit, which the
+// level-1 cubed sphere needs (160, 20 and 13 elements: its V-cycle with the CG
+// eigenvalue estimate amplifies rounding 1e8 times).
 // Up to kX64FusedMaxElems elements the degrees share one launch (960 hp elements:
-// 126 us against 251 in a launch per degree; 7,680: 642 against 571).
+// 126 us against 251 in a launch per degree; 7,680: 642 against 571; both with one
+// exponent per element).
 constexpr int kX64MinElems = 305;
 constexpr int kX64FusedMaxElems = 2048;
+// Low degrees stay native: a tile takes its time however little of it is used (a
+// face of p = 1 fills 4 of 64 points), where the native kernels' work shrinks.  The
+// line, native against digits (us): means of 17 DOFs per element (p 1..2) 66 | 86
+// on 960 elements, 273 | 323 on 7,680, 1795 | 2353 on 61,440; 33 (p 1..3) 77 | 83,
+// 330 | 338, 2209 | 2437; 45 (p 2..3) 80 | 80, 360 | 345; 56 (p 1..4) 385 | 354; 64 (p =
+// 3) 224 | 174, 1449 | 1301.  Alone on a level and not too many, p = 1 and 2 are the
+// exception: p = 1 42 | 40 at 512 elements, 129 | 157 at 4,096; p = 2 54 | 40, 175 |
+// 164, and 1079 | 1242 at 32,768.
+inline bool x64_pays(int n_elems, const BucketInfo* buckets) {
+    if (n_elems < kX64MinElems) return false;
+    long long dofs = 0;
+    int degrees = 0, top = 0;
+    for (int n = kMinN; n <= kMaxN; ++n) {
+        if (buckets[n].count == 0) continue;
+        dofs += (long long)buckets[n].count * n * n * n;
+        ++degrees;
+        top = n;
+    }
+    return dofs >= 40LL * n_elems || (degrees == 1 && n_elems <= (top == 2 ? 1024 : 4096));
+}
 cudaError_t launch_apply_x64(const LevelView<double>& L, const BucketInfo* buckets, const double* x, double* y,
                              cudaStream_t st, int* launches, const ApplyStreams* as);
 

@@ -1438,7 +1438,7 @@ template <typename T, typename TX>
 cudaError_t launch_apply_x(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y, cudaStream_t st,
                            int* launches, int* plan, const ApplyStreams* as = nullptr) {
     if constexpr (sizeof(T) == 8)
-        if (L.x64.w != nullptr && L.n_elems >= kX64MinElems && !L.bdiag && forced_plan() < 0)
+        if (L.x64.w != nullptr && !L.bdiag && forced_plan() < 0 && x64_pays(L.n_elems, buckets))
             return launch_apply_x64(L, buckets, x, y, st, launches, as);
     int path = L.n_elems <= apply_detail::kCtaMaxElems ? 0 : (L.n_elems <= apply_detail::kFusedMaxElems ? 1 : 2);
     const bool one = sizeof(T) == 4 && L.snb != nullptr;

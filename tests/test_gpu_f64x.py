@@ -101,7 +101,7 @@ def test_zeroth_order_term(name):
     assert float((y1 - y0 - F).norm()) <= 1e-12 * float(y1.norm())
 
 
-def _native(name, x, tmp_path):
+def _native(name, x, tmp_path, plan=2):
     """The same apply by the FP64 kernels (a process of its own: the plan is fixed at the first apply)."""
     here = os.path.dirname(os.path.abspath(__file__))
     np.save(tmp_path / "x.npy", x)
@@ -111,7 +111,7 @@ def _native(name, x, tmp_path):
             "np.save(sys.argv[3], np.array(y))\n")
     path = os.pathsep.join([here, os.path.dirname(here), os.environ.get("PYTHONPATH", "")])
     subprocess.run([sys.executable, "-c", code, name, str(tmp_path / "x.npy"), str(tmp_path / "y.npy")], check=True,
-                   env=dict(os.environ, DGELL_APPLY_PLAN="2", PYTHONPATH=path), cwd=os.path.dirname(here))
+                   env=dict(os.environ, DGELL_APPLY_PLAN=str(plan), PYTHONPATH=path), cwd=os.path.dirname(here))
     return np.load(tmp_path / "y.npy")
 
 
@@ -190,3 +190,16 @@ def test_non_finite_values_in_the_volume_terms(p, value):
         fin = np.isfinite(y[off[e]:off[e + 1]])
         assert fin.all() if not near[e] else not fin.all()
     assert not np.isfinite(y[off[e0]:off[e0 + 1]]).any()
+
+
+MESHES_LOW = {"p1_4096": lambda: single(1, level=4), "p1to2": lambda: inputs.sweep_mesh(level=3, pmin=1, pmax=2)}
+MESHES.update(MESHES_LOW)
+
+
+@pytest.mark.parametrize("name", list(MESHES_LOW))
+def test_low_degrees_stay_on_the_native_kernels(name, tmp_path):
+    """Bit for bit one of the native plans (which one is timed)."""
+    ctx = dgell.Context(MESHES[name]())
+    x = torch.randn(ctx.level_info()["n_dofs"], dtype=torch.float64, device="cuda")
+    y = _apply(ctx, x).cpu().numpy()
+    assert any(np.array_equal(y, _native(name, x.cpu().numpy()[None], tmp_path, plan)[0]) for plan in range(3))
