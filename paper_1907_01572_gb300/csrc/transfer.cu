@@ -61,7 +61,8 @@ __global__ void prolong_kernel(TransferView<T> t, const T* __restrict__ vH, T* _
 // interpolations run side by side (they are a chain of dependent passes, bound by
 // latency: 216 -> 27 elements, n <= 7, FP32, took 41 us one child after the other,
 // 13 us now) and are summed in child order.
-constexpr int kChildThreads = 128, kMaxChildren = 8;
+// Levels of up to kSideBySideMax coarse elements (7,680 -> 960: 39 and 27 us).
+constexpr int kChildThreads = 128, kMaxChildren = 8, kSideBySideMax = 2048;
 
 template <typename T>
 __global__ void __launch_bounds__(kChildThreads* kMaxChildren) restrict_kernel(TransferView<T> t, const T* __restrict__ rh,
@@ -97,6 +98,39 @@ __global__ void __launch_bounds__(kChildThreads* kMaxChildren) restrict_kernel(T
     }
 }
 
+// The same, one child after the other, in 128 threads: more coarse elements fill
+// the chip by themselves, and eight children's 47 KB (FP32) or 93 KB (FP64), with
+// threads that wait where an element was carried over and has one child, cost more
+// than they give (FP32, side by side and in turn: 61,440 -> 7,680 elements 161 and
+// 127 us, 32,768 -> 4,096 of p = 2 60 and 39 us).
+template <typename T>
+__global__ void __launch_bounds__(kChildThreads) restrict_in_turn_kernel(TransferView<T> t, const T* __restrict__ rh,
+                                                                         T* __restrict__ fH) {
+    constexpr int N3 = kMaxN * kMaxN * kMaxN;
+    __shared__ T b0[N3], b1[N3], acc[N3];
+    const int H = blockIdx.x, tid = threadIdx.x;
+    const int nH = t.pH[H] + 1, n3H = nH * nH * nH;
+    for (int k = tid; k < n3H; k += kChildThreads) acc[k] = 0;
+    for (int ci = t.child_off[H]; ci < t.child_off[H + 1]; ++ci) {
+        const int c = t.child_id[ci], bits = t.child_bits[ci], nh = t.ph[c] + 1;
+        const T *src = rh + t.dofh[c], *res = src;   // a carried-over element's values are copied
+        if (bits != 0xFF) {
+            for (int k = tid; k < nh * nh * nh; k += kChildThreads) b0[k] = src[k];
+            __syncthreads();
+            int d0[3] = {nh, nh, nh}, d1[3] = {nH, nh, nh}, d2[3] = {nH, nH, nh}, d3[3] = {nH, nH, nH};
+            rect_pass(b0, b1, t.tab + tab_ci(nH, nh, bits & 1), 0, nh, d0, d1, true, nH, tid, kChildThreads);
+            __syncthreads();
+            rect_pass(b1, b0, t.tab + tab_ci(nH, nh, (bits >> 1) & 1), 1, nh, d1, d2, true, nH, tid, kChildThreads);
+            __syncthreads();
+            rect_pass(b0, b1, t.tab + tab_ci(nH, nh, (bits >> 2) & 1), 2, nh, d2, d3, true, nH, tid, kChildThreads);
+            res = b1;
+        }
+        for (int k = tid; k < n3H; k += kChildThreads) acc[k] += res[k];   // (each thread its own values throughout)
+        __syncthreads();
+    }
+    for (int k = tid; k < n3H; k += kChildThreads) fH[t.dofH[H] + k] = acc[k];
+}
+
 }  // namespace
 
 template <typename T>
@@ -106,6 +140,10 @@ cudaError_t launch_prolong_add(const TransferView<T>& t, const T* vH, T* vh, cud
 }
 template <typename T>
 cudaError_t launch_restrict(const TransferView<T>& t, const T* rh, T* fH, cudaStream_t st) {
+    if (t.n_coarse > kSideBySideMax) {
+        restrict_in_turn_kernel<T><<<t.n_coarse, kChildThreads, 0, st>>>(t, rh, fH);
+        return cudaGetLastError();
+    }
     constexpr size_t smem = sizeof(T) * 2 * kMaxChildren * kMaxN * kMaxN * kMaxN;
     static const cudaError_t attr = cudaFuncSetAttribute(restrict_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess) return attr;

@@ -94,3 +94,21 @@ def test_galerkin_blocks_on_the_coarse_levels(desc):
         size = float(c1.norm()) + float(f1.norm())
         assert float((c1 - c0 - want).norm()) <= 1e-13 * size
         assert float((s1 - s0 - want).norm()) <= 1e-6 * size
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("desc", [inputs.sweep_mesh(level=5, seed=2, pmin=1, pmax=2), single(1, level=5)], ids=["hp", "p1"])
+def test_restriction_of_large_levels_is_the_transposed_prolongation(desc, dtype):
+    """f_H . v = r . (P v), with more coarse elements than run their children side by side (2,048),
+    carried-over ones among them; each product is rounded a few dozen times."""
+    ctx = dgell.Context(desc)
+    low = ctx.n_levels - 2
+    n_c, n_f = ctx.level_info(low)["n_dofs"], ctx.level_info(low + 1)["n_dofs"]
+    assert ctx.level_info(low)["n_elems"] > 2048
+    g = torch.Generator(device="cuda").manual_seed(1)
+    r = torch.randn(n_f, dtype=dtype, device="cuda", generator=g)
+    v = torch.randn(n_c, dtype=dtype, device="cuda", generator=g)
+    f = ctx.transfer(low, 1, r, torch.full_like(v, float("nan")))
+    up = ctx.transfer(low, 0, v, torch.zeros_like(r))
+    want = r.double() * up.double()
+    assert abs(float((f.double() * v.double()).sum() - want.sum())) <= 32 * torch.finfo(dtype).eps * float(want.abs().sum())
