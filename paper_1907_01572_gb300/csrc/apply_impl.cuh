@@ -1422,14 +1422,16 @@ cudaError_t launch_path(int path, const LevelView<T>& L, const BucketInfo* bucke
 // Launch plan of a level: 0 one CTA per element, 1 one warp per element in a
 // single launch per kernel, 2 per-degree-bucket launches with occupancy-sized
 // CTAs, 3 the same spread over side streams, 4 (FP32, small levels) everything
-// in one launch (apply_one.cuh).  With a plan slot and outside
-// stream capture the first apply times the candidates (each writes the same
-// outputs, in the same order of summation) and keeps the fastest; otherwise a
-// size rule picks.  DGELL_APPLY_PLAN=0..3 fixes the plan of every tuned level.
+// in one launch (apply_one.cuh).  With a plan slot and outside stream capture the
+// first apply times the candidates and keeps the fastest; otherwise a size rule
+// picks.  Results are the same from run to run of a plan; between plans only 2 and
+// 3 agree bit for bit, the others add the parts of a node in orders of their own.
+// DGELL_APPLY_PLAN=0..4 fixes the plan of every tuned level (4: of those that have
+// it; the others are tuned).
 inline int forced_plan() {
     static const int v = [] {
         const char* e = std::getenv("DGELL_APPLY_PLAN");
-        return (e && e[0] >= '0' && e[0] <= '3' && e[1] == 0) ? e[0] - '0' : -1;
+        return (e && e[0] >= '0' && e[0] <= '4' && e[1] == 0) ? e[0] - '0' : -1;
     }();
     return v;
 }
@@ -1437,15 +1439,16 @@ inline int forced_plan() {
 template <typename T, typename TX>
 cudaError_t launch_apply_x(const LevelView<T>& L, const BucketInfo* buckets, const TX* x, T* y, cudaStream_t st,
                            int* launches, int* plan, const ApplyStreams* as = nullptr) {
+    const bool one = sizeof(T) == 4 && L.snb != nullptr;
+    const int forced = forced_plan() == 4 && !one ? -1 : forced_plan();
     if constexpr (sizeof(T) == 8)
-        if (L.x64.w != nullptr && !L.bdiag && forced_plan() < 0 && x64_pays(L.n_elems, buckets))
+        if (L.x64.w != nullptr && !L.bdiag && forced < 0 && x64_pays(L.n_elems, buckets))
             return launch_apply_x64(L, buckets, x, y, st, launches, as);
     int path = L.n_elems <= apply_detail::kCtaMaxElems ? 0 : (L.n_elems <= apply_detail::kFusedMaxElems ? 1 : 2);
-    const bool one = sizeof(T) == 4 && L.snb != nullptr;
     if (one && L.n_elems <= 2 * apply_detail::kCtaMaxElems) path = 4;
     if (plan && *plan >= 0) return launch_path<T, TX>(*plan, L, buckets, x, y, st, launches, as);
-    if (plan && forced_plan() >= 0) {
-        *plan = forced_plan();
+    if (plan && forced >= 0) {
+        *plan = forced;
         return launch_path<T, TX>(*plan, L, buckets, x, y, st, launches, as);
     }
     unsigned long long key = 1469598103934665603ull;   // FNV-1a over the level shape and precision

@@ -1,7 +1,12 @@
 """FP32 apply in one launch (small levels): against the oracle over side
 degrees, hanging faces, turned blocks and coarse levels.  Which plan a level
 takes is timed, except under stream capture, where a level of up to 304
-elements takes the one-launch form: so the tests capture the apply."""
+elements takes the one-launch form, or with DGELL_APPLY_PLAN=4, read at a
+process's first apply: so the tests capture the apply or run it in a child."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -60,3 +65,47 @@ def test_captured_apply_on_coarse_levels_with_the_zeroth_order_term():
         g.replay()
         torch.cuda.synchronize()
         assert rel_l2(y.double().cpu().numpy(), y64.cpu().numpy()) < 1e-5
+
+
+def _plan4(code):
+    here = os.path.dirname(os.path.abspath(__file__))
+    path = os.pathsep.join([here, os.path.dirname(here), os.environ.get("PYTHONPATH", "")])
+    code = ("import torch\nfrom gpu_util import CASES, single, rel_l2\nfrom paper_1907_01572_gb300 import dgell, inputs\n"
+            "def randn(n):\n    return torch.tensor(inputs.random_vector(n, seed=3), device='cuda')\n" + code)
+    return subprocess.run([sys.executable, "-c", code], check=True, capture_output=True, text=True,
+                          env=dict(os.environ, DGELL_APPLY_PLAN="4", PYTHONPATH=path), cwd=os.path.dirname(here)).stdout.split()
+
+
+def test_levels_of_up_to_608_elements():
+    """512 elements of one degree and of mixed degrees, against the FP64 apply."""
+    out = _plan4("""
+for d in (single(5, level=3, warp=(0.02, (1, 2, 1))), inputs.sweep_mesh(level=3, seed=5, pmin=1, pmax=8, refine_octant=False)):
+    ctx = dgell.Context(d)
+    n = ctx.level_info()["n_dofs"]
+    assert 304 < ctx.level_info()["n_elems"] <= 608
+    for dt in (torch.float32, torch.bfloat16):
+        x = randn(n).to(dt)
+        y, want = torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda")
+        ctx.apply(x.double(), want)
+        k = ctx.launch_count()
+        ctx.apply(x, y)
+        print(ctx.launch_count() - k, rel_l2(y.double().cpu().numpy(), want.cpu().numpy()))
+""")
+    assert out[::2] == ["1"] * 4
+    assert all(float(v) < 1e-5 for v in out[1::2])   # the FP32 parity bound
+
+
+def test_element_diagonal_blocks():
+    """The smoother with element subdomains (the neighbour's traces taken as 0): FP32 against FP64 V-cycle,
+    with a fixed number of local CG steps.  FP32 rounding, amplified by the local problems' condition
+    (a few hundred), stays below 1e-3; a neighbour's trace left in would change a fifth of the values' size."""
+    out = _plan4("""
+for name in ("config1_affine_p3", "mixed_curved_2to1_l1"):
+    ctx = dgell.Context(CASES[name]())
+    f = randn(ctx.level_info()["n_dofs"])
+    v = [torch.empty_like(f, dtype=t) for t in (torch.float64, torch.float32)]
+    for w in v:
+        ctx.vcycle(f.to(w.dtype), w, smoother=1, local_iters=6, local_tol=1e-12)
+    print(rel_l2(v[1].double().cpu().numpy(), v[0].cpu().numpy()))
+""")
+    assert all(float(v) < 1e-3 for v in out) and len(out) == 2
