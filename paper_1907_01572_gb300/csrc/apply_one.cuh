@@ -239,7 +239,10 @@ __device__ __forceinline__ void one_body(const LevelView<T>& L, const ElemDesc& 
     T* F = TR + kOneMaxSlots * kOneTrace + warp * kOneScratch;
     __shared__ int next_task, face_start[7];
     const int ns = min(de.s1 - de.s0, kOneMaxSlots);
-    if (tid == 0) next_task = 0;
+    if (tid == 0) {
+        next_task = 0;
+        if (de.s1 - de.s0 > kOneMaxSlots) atomicExch(L.chk, 7);
+    }
     __syncthreads();
     if (warp < kOneVolWarps) one_volume<N, T, TX>(L, x + de.dofo, de.vo, sV, Y);
     if (warp == kOneWarps - 1) {   // first slot of each face (slots come face by face)

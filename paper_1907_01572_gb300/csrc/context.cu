@@ -1421,6 +1421,7 @@ int dg_estimate_fiducial(dg_ctx* c, const dg_block* fiducial, int n_fiducial, co
     int rc = e == cudaSuccess ? apply_t<double>(c, l, u, y) : DG_OK;   // fills the trace buffer with u's traces
     if (e == cudaSuccess && rc == DG_OK) {
         EstimateArgs a{};
+        a.chk = device_check_flag();
         a.n_elems = L.h.n_elems();
         a.p = L.p;
         a.dof_off = L.dof_off;

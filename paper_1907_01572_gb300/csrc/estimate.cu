@@ -147,7 +147,16 @@ __device__ void map_first(const dg_block& B, const double xi[3], double J[3][3],
     }
 }
 
-// S[c] = sum_i g_i d^2 x_i / dxi_l dxi_m, pairs in the order of Derivs::h.
+// S[c] = sum_i g_i d^2 x_i / dxi_l dxi_m, pairs in the order of Derivs::h: the
+// second derivatives of the formulas in block_point, for the exact Laplacian of
+// mapped polynomials.  Wedge and shell, with v linear in xi_0, xi_1, u = v / |v|,
+// t = (xi_2 + 1) / 2 and a, b in {0, 1} along e_ta:
+//   d_a u_i = (delta_i,ta - u_i u_ta) / |v|,
+//   d_a d_b u_i = -[(d_b u_i) u_ta + u_i (d_b u_ta) + (d_a u_i) u_tb] / |v|;
+//   wedge x = (1 - t) a v + t r u: d_a d_b x = t r d_a d_b u,
+//     d_a d_2 x = (r d_a u - a e_ta) / 2, d_2 d_2 x = 0;
+//   shell x = R(t) u: d_a d_b x = R d_a d_b u, d_a d_2 x = R' d_a u / 2,
+//     d_2 d_2 x = R'' u / 4, R' = R^2 (1/r1 - 1/r2), R'' = 2 R R' (1/r1 - 1/r2).
 __device__ void map_second(const dg_block& B, const double xi[3], const MapPoint& p, const double g[3], double S[6]) {
     if (B.kind == DG_BLOCK_HEX8) {
         double s01 = 0.0, s02 = 0.0, s12 = 0.0;
@@ -349,6 +358,7 @@ __global__ void __launch_bounds__(kEstThreads) estimate_kernel(EstimateArgs a, c
 
     // mortar terms of the element's slots, a warp per slot, summed in slot order
     const int s0 = a.slot_off[e], ns = a.slot_off[e + 1] - s0, lane = threadIdx.x & 31;
+    if (ns > kEstMaxSlots && threadIdx.x == 0) atomicExch(a.chk, 6);
     for (int s = threadIdx.x >> 5; s < ns && s < kEstMaxSlots; s += blockDim.x >> 5) {
         const int mi = a.slot_mortar[s0 + s];
         const Mortar Mo = a.mortars[mi];

@@ -30,6 +30,7 @@ struct EstimateArgs {
     const dg_block* fblocks;
     const double* mgW;
     const double* sigW;
+    int* chk;               // self-check flag
 };
 
 // eta2[e] = h_e^2 p_e^2 ||f u - g - Lap u||^2_e + the mortar terms of the element.
