@@ -43,14 +43,14 @@ constexpr int kOneMaxElems = 608;
 
 // FP64 with the contractions on the tensor pipe (apply_f64x.cuh): levels of at
 // least kX64MinElems elements, two per SM, where the chip is full enough for the
-// digits' throughput to count more than an element's latency (512 elements of p =
-// 3: 41 us against 64 of the native kernels; 216 are no longer two per SM).  On
-// those below, the native kernels also keep their results bit for bit, which the
-// level-1 cubed sphere needs (160, 20 and 13 elements: its V-cycle with the CG
-// eigenvalue estimate amplifies rounding 1e8 times).
+// digits' throughput to count more than an element's latency.  Native against
+// digits (us): 64 elements of p = 3 20 | 31, p = 5 35 | 56, p = 7 50 | 62; 120 hp
+// elements 68 | 62; 160 of the level-1 cubed sphere 103 | 161; 512 elements of p = 3
+// 64 | 41, p = 7 304 | 78.  (That sphere's V-cycle with the CG eigenvalue estimate
+// amplifies rounding 1e8 times; below the line its FP64 results keep their bits.)
 // Up to kX64FusedMaxElems elements the degrees share one launch (960 hp elements:
-// 126 us against 251 in a launch per degree; 7,680: 642 against 571; both with one
-// exponent per element).
+// 133 us against 299 in a launch per degree, 1,056 of the cubed sphere 303 against
+// 508; 7,680: 723 against 562).
 constexpr int kX64MinElems = 305;
 constexpr int kX64FusedMaxElems = 2048;
 // Low degrees stay native: a tile takes its time however little of it is used (a

@@ -846,7 +846,8 @@ __device__ __forceinline__ void x64_volume(const double* __restrict__ x, const d
 
 // Degrees whose volume terms stay in FP64: a pass of the integers takes the
 // time of a tile (about 1.5 us of latency) however few pencils it has, and
-// 12 n^4 FP64 multiply-adds are fewer than that up to n = 5.
+// 12 n^4 FP64 multiply-adds are fewer than that up to n = 5 (4,096 elements of p =
+// 4: 230 us, 246 on digits; 512: 50 and 56).
 template <int N>
 constexpr bool x64_small() {
     return N <= 5;
